@@ -221,8 +221,6 @@ cudaError_t launch_plain(int epi, const uint32_t *refs32, const uint32_t *ref_no
 int plain_grid_target(int epi, int device);
 cudaError_t launch_topk_merge(const uint64_t *partial, const Partition &part, int64_t n_q,
                               int32_t k, uint32_t *out_scores, int64_t *out_idx, cudaStream_t s);
-cudaError_t launch_topk_merge_tile(const uint64_t *partial, const Partition &part, int32_t tile_q, int32_t pair,
-                                   int64_t n_q, int32_t k, uint32_t *out_scores, int64_t *out_idx, cudaStream_t s);
 int64_t hits_sort_elems(int64_t capacity);
 // tensor form (tensor.cu)
 cudaError_t make_operand_map(CUtensorMap *map, const uint8_t *base, int64_t rows, int32_t kpad, int box_rows);

@@ -1,5 +1,7 @@
 // Reductions after a comparison launch: merge of per-segment top-k lists and
 // the hit-list finish (count, overflow flag, sort by (q, r)).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace fastid {
@@ -28,6 +30,39 @@ __device__ __forceinline__ uint64_t warp_merge32(uint64_t a, uint64_t b, int lan
     return v;
 }
 
+// Merge of one query's lists by W warps (a power of two, all in one block).
+// A list is k ascending keys, one per lane; list i is load(i), KEY_EMPTY on
+// lanes >= k.  Each warp folds every W-th list, MERGE_AHEAD of them loaded
+// before the first is used -- a lone warp that loaded and folded one list
+// after another was bound by that chain (0.73 us a list: 111 us for one
+// query's 149 lists, 249 us for 304) -- and a list whose smallest key cannot
+// enter is passed over.  The warps' results then meet in shared memory, in
+// log2(W) rounds.  Warp 0 of the query returns the 32 smallest keys.
+constexpr int MERGE_AHEAD = 8;
+constexpr int MERGE_MAX_WARPS = 16;
+
+template <class Load>
+__device__ __forceinline__ uint64_t merge_lists(int n, int W, int k, int lane, uint64_t (*sm)[32], Load load) {
+    const int warp = threadIdx.x >> 5, w = warp & (W - 1);
+    uint64_t acc = KEY_EMPTY;
+    for (int i = w; i < n; i += MERGE_AHEAD * W) {
+        uint64_t v[MERGE_AHEAD];
+#pragma unroll
+        for (int u = 0; u < MERGE_AHEAD; ++u) v[u] = i + u * W < n ? load(i + u * W) : KEY_EMPTY;
+#pragma unroll
+        for (int u = 0; u < MERGE_AHEAD; ++u)
+            if (shfl64(v[u], 0) < shfl64(acc, k - 1)) acc = warp_merge32(acc, v[u], lane);
+    }
+    // (a round writes rows [h, 2h) of the query's W and reads them back; the
+    // next one writes lower rows, so one barrier a round is enough)
+    for (int h = W >> 1; h > 0; h >>= 1) {
+        if (w >= h && w < 2 * h) sm[warp][lane] = acc;
+        __syncthreads();
+        if (w < h) acc = warp_merge32(acc, sm[warp + h][lane], lane);
+    }
+    return acc;
+}
+
 // CTA whose unit range contains unit u.
 __device__ int64_t cta_of(const Partition &P, int64_t u) {
     int64_t c = (u * P.grid) / P.n_units;
@@ -36,37 +71,35 @@ __device__ int64_t cta_of(const Partition &P, int64_t u) {
     return c;
 }
 
-// One warp per query: merge the sorted k-lists of every segment that covered
-// the query's tile.  The partition is over work groups (CTAs, or 2-CTA
-// clusters when paired: a paired unit covers query tiles 2 qq and 2 qq + 1,
-// taken by cluster ranks 0 and 1).  Segment lists are laid out
-// [slot][tile_q][k] with slot = cta * max_seg + (segment index within the CTA).
-__global__ void topk_merge_kernel(const uint64_t *__restrict__ partial, Partition P, int32_t tile_q, int32_t pair,
-                                  int64_t n_q, int32_t k, uint32_t *__restrict__ out_scores,
-                                  int64_t *__restrict__ out_idx) {
+// Plain launches, W warps per query: merge the sorted k-lists of every segment
+// that covered the query's tile.  Segment lists are laid out [slot][PL_TQ][k]
+// with slot = cta * max_seg + (segment index within the CTA).
+__global__ void topk_merge_kernel(const uint64_t *__restrict__ partial, Partition P, int64_t n_q, int32_t k, int W,
+                                  uint32_t *__restrict__ out_scores, int64_t *__restrict__ out_idx) {
+    __shared__ uint64_t sm[MERGE_MAX_WARPS][32];
     const int lane = threadIdx.x & 31;
-    const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (q >= n_q) return;
-    const int64_t qt = q / tile_q, ql = q - qt * tile_q;
-    const int64_t qq = pair ? qt >> 1 : qt;
-    const int64_t rank = pair ? qt & 1 : 0;
-    const int64_t u_lo = qq * P.n_rt, u_hi = u_lo + P.n_rt - 1;
-    const int64_t w_lo = cta_of(P, u_lo), w_hi = cta_of(P, u_hi);
-    uint64_t acc = KEY_EMPTY;
-    for (int64_t w = w_lo; w <= w_hi; ++w) {
-        const int64_t first_qq = part_begin(P, w) / P.n_rt;
-        const int64_t cta = pair ? 2 * w + rank : w;
-        const int64_t slot = cta * P.max_seg + (qq - first_qq);
-        uint64_t b = lane < k ? partial[(slot * tile_q + ql) * k + lane] : KEY_EMPTY;
-        acc = warp_merge32(acc, b, lane);
+    const int warp = threadIdx.x >> 5;
+    const int64_t q = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) / W;
+    int64_t ql = 0, c_lo = 0, c_hi = -1, seg_lo = 0;
+    if (q < n_q) {
+        const int64_t qt = q / PL_TQ;
+        ql = q - qt * PL_TQ;
+        c_lo = cta_of(P, qt * P.n_rt);
+        c_hi = cta_of(P, qt * P.n_rt + P.n_rt - 1);
+        seg_lo = qt - part_begin(P, c_lo) / P.n_rt;
     }
-    if (lane < k) {
+    // (only the first CTA can have had an earlier tile: every other one starts inside this tile, segment 0)
+    const uint64_t acc = merge_lists((int)(c_hi - c_lo + 1), W, k, lane, sm, [&](int i) {
+        const int64_t slot = (c_lo + i) * P.max_seg + (i == 0 ? seg_lo : 0);
+        return lane < k ? partial[(slot * PL_TQ + ql) * k + lane] : KEY_EMPTY;
+    });
+    if (q < n_q && (warp & (W - 1)) == 0 && lane < k) {
         out_scores[q * k + lane] = acc == KEY_EMPTY ? 0xFFFFFFFFu : (uint32_t)(acc >> 32);
         out_idx[q * k + lane] = acc == KEY_EMPTY ? -1ll : (int64_t)(uint32_t)acc;
     }
 }
 
-// Tensor launches: one warp per query; its tile's lists sit in one slot of
+// Tensor launches: W warps per query; its tile's lists sit in one slot of
 // every reference slice's group of its tile group (see TcSched).  Slot
 // layout [slot][k][128].
 struct MergeSched {
@@ -103,14 +136,20 @@ __device__ __forceinline__ bool merge_slot_ok(const MergeSched &M, int64_t slot)
 }
 
 __global__ void topk_merge_sched_kernel(const uint64_t *__restrict__ partial, const MergeSched M,
-                                        const MergeJob *__restrict__ jobs, int64_t n_jobs,
+                                        const MergeJob *__restrict__ jobs, int64_t n_jobs, int W,
                                         uint32_t *__restrict__ out_s, int64_t *__restrict__ out_i) {
+    __shared__ uint64_t sm[MERGE_MAX_WARPS][32];
     const int lane = threadIdx.x & 31;
-    const int64_t j = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (j >= n_jobs) return;
+    const int warp = threadIdx.x >> 5;
+    const int64_t j = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) / W;
     const int k = M.k;
     MergeJob jb;
-    if (jobs) {
+    if (j >= n_jobs) {  // an idle warp of the last block: no lists, but the block's barriers
+        jb.out_s = nullptr;
+        jb.out_i = nullptr;
+        jb.panel = 0;
+        jb.q = 0;
+    } else if (jobs) {
         jb = jobs[j];
     } else {
         jb.out_s = out_s + j * k;
@@ -123,21 +162,21 @@ __global__ void topk_merge_sched_kernel(const uint64_t *__restrict__ partial, co
     const int64_t qq = M.pair ? qt >> 1 : qt;
     const int64_t rank = M.pair ? qt & 1 : 0;
     const int64_t x = qq / sc.tpx, li = qq - x * sc.tpx;
-    uint64_t acc = KEY_EMPTY;
-    for (int64_t y = 0; y < sc.b; ++y) {
-        const int64_t wg = x * sc.b + y;
-        const int64_t cta = M.pair ? 2 * wg + rank : wg;
-        const int64_t slot = (int64_t)sc.slot0 + cta * sc.tpx + li;
-        uint64_t v = lane < k && merge_slot_ok(M, slot) ? partial[(slot * k + lane) * TC_TILE_Q + ql] : KEY_EMPTY;
-        acc = warp_merge32(acc, v, lane);
-    }
-    if (sc.t_groups > 0) {  // the tail group holding this query tile (see TcSched)
-        const int64_t cpg = M.pair ? 2 : 1;
-        const int64_t t = qq / sc.t_tpx, lt = qq - t * sc.t_tpx;
-        const int64_t slot = (int64_t)sc.slot0 + (int64_t)sc.a * sc.b * cpg * sc.tpx + (t * cpg + rank) * sc.t_tpx + lt;
-        uint64_t v = lane < k && merge_slot_ok(M, slot) ? partial[(slot * k + lane) * TC_TILE_Q + ql] : KEY_EMPTY;
-        acc = warp_merge32(acc, v, lane);
-    }
+    const int64_t cpg = M.pair ? 2 : 1;
+    // lists 0 .. b - 1: the slices' groups; list b: the tail group holding
+    // this query tile, if there is a tail (see TcSched)
+    const int n = j < n_jobs ? sc.b + (sc.t_groups > 0 ? 1 : 0) : 0;
+    uint64_t acc = merge_lists(n, W, k, lane, sm, [&](int i) {
+        int64_t slot;
+        if (i < sc.b) {
+            slot = (int64_t)sc.slot0 + ((x * sc.b + i) * cpg + rank) * sc.tpx + li;
+        } else {
+            const int64_t t = qq / sc.t_tpx, lt = qq - t * sc.t_tpx;
+            slot = (int64_t)sc.slot0 + (int64_t)sc.a * sc.b * cpg * sc.tpx + (t * cpg + rank) * sc.t_tpx + lt;
+        }
+        return lane < k && merge_slot_ok(M, slot) ? partial[(slot * k + lane) * TC_TILE_Q + ql] : KEY_EMPTY;
+    });
+    if (j >= n_jobs || (warp & (W - 1)) != 0) return;
     if (M.accumulate) {
         // keys are (score << 32) | r: the offset moves r, never the score (r + offset < 2^32)
         if (acc != KEY_EMPTY) acc += (uint64_t)M.ref_offset;
@@ -326,23 +365,29 @@ int64_t hits_sort_elems(int64_t capacity) {
     return p < SB ? SB : p;
 }
 
+// Warps per query for n_q queries of up to n lists: about MERGE_AHEAD lists a
+// warp, so that one round of loads covers them, but no more warps than about
+// two waves of the GPU's (152 SMs x 64): past that more warps a query only
+// add shared-memory rounds (7165 queries of a 4-panel plan, up to 76 lists:
+// 52 us with 16 warps each; one warp a query took 33 us).  One query of 149
+// lists: 111 -> 8.9 us; 48 of 152: 119 -> 8.8; 32 of 304 (plain): 249 -> 11.7;
+// 2048 of 10: 11.5 -> 10.5.
+static int merge_warps(int64_t n_q, int64_t n_lists) {
+    int W = 1;
+    while (W < MERGE_MAX_WARPS && (int64_t)W * MERGE_AHEAD < n_lists && 2 * W * n_q <= 16384) W <<= 1;
+    return W;
+}
+
+// Blocks of 8 warps, or of W where a query takes more.
+static int merge_block_warps(int W) { return W > 8 ? W : 8; }
+
 cudaError_t launch_topk_merge(const uint64_t *partial, const Partition &part, int64_t n_q, int32_t k,
                               uint32_t *out_scores, int64_t *out_idx, cudaStream_t s) {
     if (n_q == 0) return cudaSuccess;
-    const int wpb = 8;
-    int64_t blocks = (n_q + wpb - 1) / wpb;
-    topk_merge_kernel<<<(unsigned)blocks, wpb * 32, 0, s>>>(partial, part, PL_TQ, 0, n_q, k, out_scores, out_idx);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_topk_merge_tile(const uint64_t *partial, const Partition &part, int32_t tile_q, int32_t pair,
-                                   int64_t n_q, int32_t k, uint32_t *out_scores, int64_t *out_idx,
-                                   cudaStream_t s) {
-    if (n_q == 0) return cudaSuccess;
-    const int wpb = 8;
-    int64_t blocks = (n_q + wpb - 1) / wpb;
-    topk_merge_kernel<<<(unsigned)blocks, wpb * 32, 0, s>>>(partial, part, tile_q, pair, n_q, k, out_scores,
-                                                            out_idx);
+    const int64_t n_qt = (n_q + PL_TQ - 1) / PL_TQ;
+    const int W = merge_warps(n_q, (part.grid + n_qt - 1) / n_qt + 1), per = merge_block_warps(W) / W;
+    topk_merge_kernel<<<(unsigned)((n_q + per - 1) / per), per * W * 32, 0, s>>>(partial, part, n_q, k, W, out_scores,
+                                                                                out_idx);
     return cudaGetLastError();
 }
 
@@ -360,9 +405,12 @@ cudaError_t launch_merge_sched(const uint64_t *partial, const TcLaunch &L, const
     M.n_slots = L.n_slots;
     M.status = L.status;
     M.qspread = L.qspread[0];
-    const int wpb = 8;
-    int64_t blocks = (n_jobs + wpb - 1) / wpb;
-    topk_merge_sched_kernel<<<(unsigned)blocks, wpb * 32, 0, s>>>(partial, M, jobs, n_jobs, out_scores, out_idx);
+    int64_t n_lists = 1;
+    for (int p = 0; p < L.n_panels; ++p)
+        n_lists = std::max<int64_t>(n_lists, L.sched[p].b + (L.sched[p].t_groups > 0 ? 1 : 0));
+    const int W = merge_warps(n_jobs, n_lists), per = merge_block_warps(W) / W;
+    topk_merge_sched_kernel<<<(unsigned)((n_jobs + per - 1) / per), per * W * 32, 0, s>>>(partial, M, jobs, n_jobs, W,
+                                                                                         out_scores, out_idx);
     return cudaGetLastError();
 }
 
