@@ -58,6 +58,12 @@ __host__ __device__ constexpr uint32_t pk_stage_bytes(int bn, bool f4) { return 
 constexpr int TC_BN4 = 224;
 constexpr uint32_t TC_SF_COL = 448;
 constexpr uint32_t TC_SF_UNIT = 0x7F7F7F7Fu;  // four ue8m0 bytes of 2^0
+// Full-matrix launches: each epilogue warp turns a 32 x 32 block of scores
+// from thread-per-query to query-major through a buffer of 32 rows of 36
+// words (16-byte rows; a quarter-warp's 16-byte accesses meet every bank once
+// both ways).
+constexpr int SC_LD = 36;
+constexpr uint32_t SC_BYTES = 4 * 32 * SC_LD * 4;
 constexpr uint64_t WAIT_NS = 2000000000ull;     // 2 s per wait
 constexpr uint64_t RENDEZVOUS_NS = 50000000ull;  // 50 ms per panel entry, then go on alone
 
@@ -71,9 +77,12 @@ constexpr uint64_t RENDEZVOUS_NS = 50000000ull;  // 50 ms per panel entry, then 
 //   BN = 128: 16 KB reference stage, 6 stages, 2 x 128 TMEM columns
 //   CG2 (2-SM MMA, see tensor_kernel): each CTA holds half of every reference
 //             stage, 7 stages (FP8 32 KB, FP4 30 KB a stage)
-template <int BN, bool PK = false, bool CG2 = false>
+//   SC (full-matrix launches): one stage less where the transpose buffers
+//   (SC_BYTES) would not fit beside the ring
+template <int BN, bool PK = false, bool CG2 = false, bool SC = false>
 struct TcShape {
-    static constexpr int STAGES = CG2 ? 7 : BN == 128 ? 6 : (BN == 224 && !PK) ? 5 : 4;
+    static constexpr int RING = CG2 ? 7 : BN == 128 ? 6 : (BN == 224 && !PK) ? 5 : 4;
+    static constexpr int STAGES = RING - (SC && (BN == 224) != PK ? 1 : 0);
     static constexpr uint32_t B_BYTES = (uint32_t)(CG2 ? BN / 2 : BN) * TC_BK;
     static constexpr uint32_t TMEM_COLS = BN == 128 ? 256 : 512;
 };
@@ -439,6 +448,74 @@ __device__ __noinline__ void append_hit(unsigned long long *count, int64_t capac
     }
 }
 
+// Writes a warp's 32 x 32 block of full-matrix scores (v: lane's operand row,
+// 32 columns) with rows of the output written whole.  Each lane storing its
+// own row touched 32 rows an instruction, 2 or 4 useful bytes of every
+// 32-byte sector; through the transpose buffer an instruction writes whole
+// 64-byte (uint16) or 128-byte (uint32) row segments (500 x 60,001 uint32 at
+// N = 1500, 120 MB: 209 -> 56 us a call): 16-byte stores where every row
+// starts on a 16-byte boundary (vec), else a column a lane.
+// out: the block's first element; row_step: bytes between the warp's rows;
+// rows, cols: live rows and columns.  One warp a scheduler issues all of it,
+// so the loops carry pointers instead of indices (108 us with an index and a
+// bounds check a row), and the score leaves FP32 as the low bits of
+// score + 2^23 (exact: 0 <= score <= 65536).
+template <int ESZ>
+__device__ __forceinline__ void store_scores(uint8_t *out, int64_t row_step, int rows, int cols, bool vec,
+                                             uint32_t *buf, const uint32_t (&v)[32], float cq, int lane) {
+    constexpr uint32_t MAGIC = 0x4B000000u;  // 2^23
+    const float cm = cq + __uint_as_float(MAGIC);
+    __syncwarp();  // the previous block's reads are done
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) {
+        uint4 o;
+        o.x = __float_as_uint(__uint_as_float(v[j]) + cm) - MAGIC;
+        o.y = __float_as_uint(__uint_as_float(v[j + 1]) + cm) - MAGIC;
+        o.z = __float_as_uint(__uint_as_float(v[j + 2]) + cm) - MAGIC;
+        o.w = __float_as_uint(__uint_as_float(v[j + 3]) + cm) - MAGIC;
+        *reinterpret_cast<uint4 *>(buf + lane * SC_LD + j) = o;
+    }
+    __syncwarp();
+    if (vec && cols >= 32) {
+        constexpr int LPR = 2 * ESZ;       // lanes a row segment of 16-byte stores
+        constexpr int RPI = 32 / LPR;      // rows an instruction
+        const int r0 = lane / LPR, c = lane % LPR;
+        uint8_t *p = out + r0 * row_step + c * 16;
+        const uint32_t *b = buf + r0 * SC_LD + c * (16 / ESZ);
+#pragma unroll
+        for (int i = 0; i < 32 / RPI; ++i) {
+            if (r0 + i * RPI < rows) {
+                uint4 x = *reinterpret_cast<const uint4 *>(b + i * RPI * SC_LD);
+                if (ESZ == 2) {
+                    const uint4 y = *reinterpret_cast<const uint4 *>(b + i * RPI * SC_LD + 4);
+                    x = make_uint4(x.x | (x.y << 16), x.z | (x.w << 16), y.x | (y.y << 16), y.z | (y.w << 16));
+                }
+                *reinterpret_cast<uint4 *>(p) = x;
+            }
+            p += RPI * row_step;
+        }
+    } else if (lane < cols) {
+        uint8_t *p = out + lane * ESZ;
+        const uint32_t *b = buf + lane;
+        if (rows == 32) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i, p += row_step) {
+                if (ESZ == 2)
+                    *reinterpret_cast<uint16_t *>(p) = (uint16_t)b[i * SC_LD];
+                else
+                    *reinterpret_cast<uint32_t *>(p) = b[i * SC_LD];
+            }
+        } else {
+            for (int i = 0; i < rows; ++i, p += row_step) {
+                if (ESZ == 2)
+                    *reinterpret_cast<uint16_t *>(p) = (uint16_t)b[i * SC_LD];
+                else
+                    *reinterpret_cast<uint32_t *>(p) = b[i * SC_LD];
+            }
+        }
+    }
+}
+
 // Bounded wait that ignores the abort flag: used to drain this CTA's own
 // asynchronous copies and MMAs before it exits.
 __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity, uint32_t *status, uint32_t site) {
@@ -634,10 +711,13 @@ __device__ __forceinline__ void expand_stage_f4(const uint8_t *sp, uint8_t *sb, 
 // which leaves room for 7 stages.  Both CTAs' loads complete on the even
 // CTA's full barrier; its commits release both CTAs' stages and accumulators;
 // both epilogues release an accumulator on the even CTA's barrier.
-template <int BN, bool PAIR, int KM, bool PK, bool F4, bool CG2 = false>
+// SC: full-matrix launches (EPI_SCORES*), with the transpose buffers of
+// store_scores; the others filter into top-k lists (EPI_TOPK) or hits.
+template <int BN, bool PAIR, int KM, bool PK, bool F4, bool CG2 = false, bool SC = false>
 __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS, 1)
     tensor_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TensorArgs args) {
-    using S = TcShape<BN, PK, CG2>;
+    using S = TcShape<BN, PK, CG2, SC>;
+    static_assert(!SC || (KM == 16 && !CG2 && BN != 128), "full-matrix launches: the single-call shapes");
     static_assert(!CG2 || (PAIR && !PK), "2-SM MMA launches are paired, over an operand copy");
     static_assert(F4 ? BN == TC_BN4 : BN != TC_BN4, "FP4 launches use 224-reference tiles, FP8 ones 256 or 128");
     static_assert(!PAIR || BN != 128, "paired launches use 256- or 224-reference tiles");
@@ -652,7 +732,8 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
     uint8_t *sA = base;
     uint8_t *sB = base + S::STAGES * TC_A_BYTES;
     uint8_t *sP = base + S::STAGES * (TC_A_BYTES + S::B_BYTES);  // PK only
-    TcSmem *ctl = reinterpret_cast<TcSmem *>(sP + (PK ? S::STAGES * P_BYTES : 0));
+    uint8_t *sT = sP + (PK ? S::STAGES * P_BYTES : 0);  // SC only
+    TcSmem *ctl = reinterpret_cast<TcSmem *>(sT + (SC ? SC_BYTES : 0));
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -921,7 +1002,10 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
         const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
         const float tplus1 = args.threshold == 0xFFFFFFFFu ? __int_as_float(0x7f800000) : (float)args.threshold + 1.0f;
         const int k = args.k;
-        const bool topk = args.epi == EPI_TOPK;
+        const bool topk = !SC && args.epi == EPI_TOPK;
+        // every row of the output starts on a 16-byte boundary
+        const bool vec = SC && (reinterpret_cast<uintptr_t>(args.out) & 15) == 0 &&
+                         ((args.ld_out * (args.epi == EPI_SCORES16 ? 2 : 4)) & 15) == 0;
         int acc = 0;
         uint32_t acc_phase = 0;
         int32_t ls[KM];   // this thread's top-k scores (see net_insert)
@@ -942,6 +1026,18 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                     const bool qvalid = q < P.n_q;
                     const float cq = P.qconst[qr];
                     const float cut0 = qvalid ? tplus1 - cq : -__int_as_float(0x7f800000);
+                    // SC: the warp's output rows are q0, q0 + st, q0 + 2 st, ... (see spread_row_to_query)
+                    uint8_t *sc_out = nullptr;
+                    int64_t sc_step = 0;
+                    int sc_rows = 0;
+                    if constexpr (SC) {
+                        const int64_t q0 = spread_row_to_query(qt * TC_BM + quad * 32, P.qspread);
+                        const int64_t st = P.qspread <= 1 ? 1 : P.qspread;
+                        const int64_t esz = args.epi == EPI_SCORES16 ? 2 : 4;
+                        sc_rows = q0 < P.n_q ? (int)min((int64_t)32, (P.n_q - q0 + st - 1) / st) : 0;
+                        sc_out = reinterpret_cast<uint8_t *>(args.out) + q0 * args.ld_out * esz;
+                        sc_step = st * args.ld_out * esz;
+                    }
                     uint64_t *slot = args.partial + (W.slot + (qq - W.q_lo)) * (int64_t)k * TC_BM + row;
                     if (topk && rc > W.r_lo) {
                         list_load(slot, ls, lr, k);
@@ -969,20 +1065,14 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                             __syncwarp();  // tcgen05.ld is warp-collective: reconverge first
                             tmem_ld32(taddr + ch * 32, v);
                             const int64_t rch = r0 + ch * 32;
-                            if (args.epi == EPI_SCORES16 || args.epi == EPI_SCORES32) {
-                                if (qvalid) {
-#pragma unroll
-                                    for (int j = 0; j < 32; ++j) {
-                                        const int64_t r = rch + j;
-                                        if (r < n_refs) {
-                                            const uint32_t sc = (uint32_t)(int32_t)(__uint_as_float(v[j]) + cq);
-                                            if (args.epi == EPI_SCORES16)
-                                                reinterpret_cast<uint16_t *>(args.out)[q * args.ld_out + r] =
-                                                    (uint16_t)sc;
-                                            else
-                                                reinterpret_cast<uint32_t *>(args.out)[q * args.ld_out + r] = sc;
-                                        }
-                                    }
+                            if constexpr (SC) {
+                                const int cols = (int)min((int64_t)32, n_refs - rch);
+                                if (sc_rows > 0 && cols > 0) {
+                                    uint32_t *buf = reinterpret_cast<uint32_t *>(sT) + quad * 32 * SC_LD;
+                                    if (args.epi == EPI_SCORES16)
+                                        store_scores<2>(sc_out + rch * 2, sc_step, sc_rows, cols, vec, buf, v, cq, lane);
+                                    else
+                                        store_scores<4>(sc_out + rch * 4, sc_step, sc_rows, cols, vec, buf, v, cq, lane);
                                 }
                                 continue;
                             }
@@ -1251,10 +1341,11 @@ __global__ void prep_jobs_kernel(const PrepJob *__restrict__ jobs, int64_t n_job
     }
 }
 
-template <int BN, bool PK = false, bool CG2 = false>
+template <int BN, bool PK = false, bool CG2 = false, bool SC = false>
 size_t tensor_smem(bool f4 = false) {
-    using S = TcShape<BN, PK, CG2>;
-    return 1024 + S::STAGES * (size_t)(TC_A_BYTES + S::B_BYTES + (PK ? pk_stage_bytes(BN, f4) : 0)) + 256;
+    using S = TcShape<BN, PK, CG2, SC>;
+    return 1024 + S::STAGES * (size_t)(TC_A_BYTES + S::B_BYTES + (PK ? pk_stage_bytes(BN, f4) : 0)) +
+           (SC ? SC_BYTES : 0) + 256;
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link
@@ -1401,12 +1492,12 @@ int tensor_grid_target(int device) {
 
 namespace {
 
-// One launch of tensor_kernel<BN, PAIR, KM, PK, F4, CG2> over n_groups work
+// One launch of tensor_kernel<BN, PAIR, KM, PK, F4, CG2, SC> over n_groups work
 // groups (2-CTA clusters when paired).
-template <int BN, bool PAIR, int KM, bool PK = false, bool F4 = false, bool CG2 = false>
+template <int BN, bool PAIR, int KM, bool PK = false, bool F4 = false, bool CG2 = false, bool SC = false>
 cudaError_t launch_variant(const TcMaps &maps, const TensorArgs &a, int32_t n_groups, int epi, cudaStream_t s) {
-    const size_t smem = tensor_smem<BN, PK, CG2>(F4);
-    cudaError_t e = cudaFuncSetAttribute(tensor_kernel<BN, PAIR, KM, PK, F4, CG2>,
+    const size_t smem = tensor_smem<BN, PK, CG2, SC>(F4);
+    cudaError_t e = cudaFuncSetAttribute(tensor_kernel<BN, PAIR, KM, PK, F4, CG2, SC>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
@@ -1422,7 +1513,7 @@ cudaError_t launch_variant(const TcMaps &maps, const TensorArgs &a, int32_t n_gr
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = PAIR ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, tensor_kernel<BN, PAIR, KM, PK, F4, CG2>, maps, a);
+    return cudaLaunchKernelEx(&cfg, tensor_kernel<BN, PAIR, KM, PK, F4, CG2, SC>, maps, a);
 }
 
 }  // namespace
@@ -1460,6 +1551,16 @@ cudaError_t launch_tensor_multi(int bn, const TcLaunch &L, cudaStream_t s) {
     a.partial = L.partial;
     a.status = L.status;
     a.arrive = L.arrive;
+    if (L.epi == EPI_SCORES16 || L.epi == EPI_SCORES32) {
+        if (L.cg2 || (L.pk && L.pair) || (!L.f4 && bn != 256)) return cudaErrorInvalidValue;
+        if (L.f4)
+            return L.pk     ? launch_variant<TC_BN4, false, 16, true, true, false, true>(maps, a, L.n_groups, L.epi, s)
+                   : L.pair ? launch_variant<TC_BN4, true, 16, false, true, false, true>(maps, a, L.n_groups, L.epi, s)
+                            : launch_variant<TC_BN4, false, 16, false, true, false, true>(maps, a, L.n_groups, L.epi, s);
+        return L.pk     ? launch_variant<256, false, 16, true, false, false, true>(maps, a, L.n_groups, L.epi, s)
+               : L.pair ? launch_variant<256, true, 16, false, false, false, true>(maps, a, L.n_groups, L.epi, s)
+                        : launch_variant<256, false, 16, false, false, false, true>(maps, a, L.n_groups, L.epi, s);
+    }
     // 16-slot lists when k allows (half the insert network, 32 fewer registers)
     const bool k16 = L.epi != EPI_TOPK || L.k <= 16;
     if (L.f4) {  // 224-reference tiles whatever bn says
