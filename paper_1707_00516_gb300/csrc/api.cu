@@ -514,7 +514,7 @@ struct TensorPrep {
     int64_t n_ctas;
 };
 
-enum ExtraKind { EXTRA_NONE, EXTRA_TOPK, EXTRA_HITS };
+enum ExtraKind { EXTRA_NONE, EXTRA_TOPK };
 
 // op (an operand other than OP_PLAIN): FP8 or FP4 operands; packed rows
 // expanded on chip are unpaired, and their FP8 queries are encoded at half
@@ -545,7 +545,6 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
     tp->n_ctas = (int64_t)L.n_groups * (L.pair ? 2 : 1);
     size_t extra = 0;
     if (ek == EXTRA_TOPK) extra = (size_t)L.n_slots * tensor_tile_q() * (size_t)karg * 8;
-    if (ek == EXTRA_HITS) extra = 256 + (size_t)(2 + hits_sort_elems(karg) * 3 / 2 + 1) * 8;
     Carver cv;
     size_t o_a = cv.take<uint8_t>((size_t)n_q_pad * kbytes);
     size_t o_c = cv.take<float>((size_t)n_q_pad);
@@ -759,17 +758,17 @@ fastid_status fastid_compare(fastid_ctx *ctx, const fastid_refdb *db, const uint
         return FASTID_OK;
     }
     // device hit counter and the sort's scratch
+    const int passes = hits_passes(n_q, db->n_refs);
+    const HitsLayout HL = hits_layout(capacity, passes);
     Scratch aux(ctx, s);
-    FASTID_CUDA(ctx, aux.alloc(fastid::hits_aux_bytes(capacity)));
-    unsigned long long *count = at<unsigned long long>(aux.p, 0);
-    uint64_t *sort_tmp = at<uint64_t>(aux.p, 256);
-    FASTID_CUDA(ctx, cudaMemsetAsync(count, 0, sizeof(unsigned long long), s));
+    FASTID_CUDA(ctx, aux.alloc(HL.bytes));
+    FASTID_CUDA(ctx, cudaMemsetAsync(aux.p, 0, HL.zero_bytes, s));
     if ((st = fastid::compare_append(ctx, db, queries_dev, ld_q, n_q, modes_dev, threshold, capacity, hit_q_dev,
-                                     hit_r_dev, hit_score_dev, count, s)))
+                                     hit_r_dev, hit_score_dev, at<unsigned long long>(aux.p, 0), s)))
         return st;
-    FASTID_CUDA(ctx, launch_hits_finish(count, capacity, hit_q_dev, hit_r_dev, hit_score_dev, hit_count_dev, sort_tmp,
-                                        ctx->dev_status, s));
-    count_launches(ctx, hits_finish_launches(capacity));
+    FASTID_CUDA(ctx, launch_hits_finish(aux.p, capacity, n_q, db->n_refs, hit_q_dev, hit_r_dev, hit_score_dev,
+                                        hit_count_dev, ctx->dev_status, s));
+    count_launches(ctx, hits_finish_launches(capacity, passes));
     return FASTID_OK;
 }
 
@@ -825,10 +824,6 @@ int pick_operand(int form, bool has_fp8, bool has_fp4, int64_t n_q, bool slots16
     }
 }
 
-size_t hits_aux_bytes(int64_t capacity) {
-    return 256 + (size_t)(2 + hits_sort_elems(capacity) * 3 / 2 + 1) * 8;
-}
-
 fastid_status compare_append(fastid_ctx *ctx, const fastid_refdb *db, const uint64_t *queries_dev, int64_t ld_q,
                              int64_t n_q, const uint8_t *modes_dev, uint32_t threshold, int64_t capacity,
                              int64_t *hit_q_dev, int64_t *hit_r_dev, uint32_t *hit_score_dev,
@@ -870,14 +865,6 @@ fastid_status compare_append(fastid_ctx *ctx, const fastid_refdb *db, const uint
     return FASTID_OK;
 }
 
-int64_t hits_finish_launches(int64_t capacity) {
-    if (capacity == 0) return 1;
-    int64_t P = hits_sort_elems(capacity), n = 4;  // prep, keys, first smem sort, unpack
-    for (int64_t size = 2 * 2048; size <= P; size <<= 1) {
-        for (int64_t j = size >> 1; j >= 2048; j >>= 1) ++n;
-        ++n;
-    }
-    return n;
-}
+int64_t hits_finish_launches(int64_t capacity, int passes) { return capacity == 0 ? 1 : 1 + passes; }
 
 }  // namespace fastid

@@ -221,7 +221,15 @@ cudaError_t launch_plain(int epi, const uint32_t *refs32, const uint32_t *ref_no
 int plain_grid_target(int epi, int device);
 cudaError_t launch_topk_merge(const uint64_t *partial, const Partition &part, int64_t n_q,
                               int32_t k, uint32_t *out_scores, int64_t *out_idx, cudaStream_t s);
-int64_t hits_sort_elems(int64_t capacity);
+// Hit-list finish (reduce.cu).  The scratch of a hit call holds the device
+// counter, the sort's digit tables (zero_bytes from the start are zero before
+// the call's first kernel) and its key and score arrays.
+struct HitsLayout {
+    size_t table, keys, vals;  // offsets
+    size_t zero_bytes, bytes;
+};
+int hits_passes(int64_t n_q, int64_t n_refs);  // sort passes, even
+HitsLayout hits_layout(int64_t capacity, int passes);
 // tensor form (tensor.cu)
 cudaError_t make_operand_map(CUtensorMap *map, const uint8_t *base, int64_t rows, int32_t kpad, int box_rows);
 int tensor_tile_q();
@@ -265,7 +273,9 @@ cudaError_t launch_merge_sched(const uint64_t *partial, const TcLaunch &L, const
 // running [n_q][k] lists.
 cudaError_t launch_topk_fold(uint32_t *run_s, int64_t *run_i, const uint32_t *blk_s, const int64_t *blk_i,
                              int64_t offset, int64_t n_q, int32_t k, cudaStream_t s);
-cudaError_t launch_hits_finish(unsigned long long *count, int64_t capacity, int64_t *hit_q,
-                               int64_t *hit_r, uint32_t *hit_score, int64_t *count_out,
-                               uint64_t *sort_tmp, uint32_t *status, cudaStream_t s);
+// Sorts the hits appended under the counter at aux (see HitsLayout) by (q, r),
+// for 0 <= q < n_q and 0 <= r < n_refs; writes the true count.
+cudaError_t launch_hits_finish(void *aux, int64_t capacity, int64_t n_q, int64_t n_refs, int64_t *hit_q,
+                               int64_t *hit_r, uint32_t *hit_score, int64_t *count_out, uint32_t *status,
+                               cudaStream_t s);
 }  // namespace fastid

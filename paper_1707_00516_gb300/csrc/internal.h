@@ -114,10 +114,8 @@ fastid_status compare_append(fastid_ctx *ctx, const fastid_refdb *db, const uint
                              int64_t n_q, const uint8_t *modes_dev, uint32_t threshold, int64_t capacity,
                              int64_t *hit_q_dev, int64_t *hit_r_dev, uint32_t *hit_score_dev,
                              unsigned long long *count, cudaStream_t s);
-// Bytes of a hit call's counter (at 0) and sort scratch (at 256).
-size_t hits_aux_bytes(int64_t capacity);
-// Kernel launches of launch_hits_finish for this capacity.
-int64_t hits_finish_launches(int64_t capacity);
+// Kernel launches of launch_hits_finish.
+int64_t hits_finish_launches(int64_t capacity, int passes);
 // Streamed blocks, hit lists: snaps[b] = *count, then hits appended by block
 // b (since snaps[b - 1]) get r0 added to their reference index (2 launches,
 // or 1 when r0 == 0).  In reduce.cu.

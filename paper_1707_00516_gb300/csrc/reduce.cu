@@ -235,134 +235,204 @@ __global__ void hits_offset_kernel(const unsigned long long *__restrict__ snaps,
 }
 
 // ---- hit list finish ----------------------------------------------------
-// sort_tmp layout: [0] = live count n (as u64), [1] = next power of two of n,
-// then keys[P], then vals (u32)[P].
+// The list is sorted by (q, r) with a least-significant-digit radix sort on
+// the key q << r_bits | r, in an even number of passes so that it leaves the
+// caller's buffers for the scratch arrays and ends in them.  A block takes
+// 2^rs_shift consecutive elements (at least RS_TILE, at most RS_BLOCKS
+// blocks); table[p][block][digit] holds each block's digit counts for pass p,
+// counted by a kernel of its own for the first pass and by the previous
+// pass's scatter (which knows every element's place in the next order) for
+// the others, so that a pass is one launch.  Everything is sized on the device
+// by the live count.  (A bitonic sort over the buffer's capacity took 57
+// launches and ~240 us for 60,000 hits in a buffer of 2^20, 1 ms in one of
+// 2^21, whatever the count; the count kernel and four passes take ~53 us, half
+// of it the global atomics of the next counts: a kernel of its own for those
+// would cost as much.)
+constexpr int RS_BITS = 8;
+constexpr int RS_DIGITS = 1 << RS_BITS;
+constexpr int RS_THREADS = 1024;
+constexpr int RS_ITEMS = 4;  // elements a thread
+constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
+constexpr int RS_WARPS = RS_THREADS / 32;
+constexpr int RS_GROUPS = RS_THREADS / RS_DIGITS;
+constexpr int RS_BLOCKS = 256;  // about what fits the GPU at once (two a SM); every block reads every block's counts
 
-__global__ void hits_prep_kernel(const unsigned long long *__restrict__ count, int64_t capacity,
-                                 int64_t *__restrict__ count_out, uint64_t *__restrict__ tmp,
-                                 uint32_t *__restrict__ status) {
-    unsigned long long c = *count;
-    unsigned long long n = c < (unsigned long long)capacity ? c : (unsigned long long)capacity;
-    unsigned long long p = 1;
-    while (p < n) p <<= 1;
-    tmp[0] = n;
-    tmp[1] = p;
-    *count_out = (int64_t)c;
-    if (c > (unsigned long long)capacity) atomicOr(status, ST_OVERFLOW);
+__device__ __forceinline__ int64_t hits_live(const unsigned long long *count, int64_t capacity) {
+    const unsigned long long c = *count;
+    return (int64_t)(c < (unsigned long long)capacity ? c : (unsigned long long)capacity);
 }
 
-__global__ void hits_keys_kernel(const int64_t *__restrict__ hq, const int64_t *__restrict__ hr,
-                                 const uint32_t *__restrict__ hs, uint64_t *__restrict__ tmp, int64_t P) {
-    const uint64_t n = tmp[0], pn = tmp[1];
-    uint64_t *keys = tmp + 2;
-    uint32_t *vals = reinterpret_cast<uint32_t *>(tmp + 2 + P);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)pn;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if ((uint64_t)i < n) {
-            keys[i] = ((uint64_t)hq[i] << 32) | (uint64_t)(uint32_t)hr[i];
-            vals[i] = hs[i];
-        } else {
-            keys[i] = KEY_EMPTY;
-            vals[i] = 0;
-        }
+// log2 of a block's elements
+__device__ __forceinline__ int rs_shift(int64_t n) {
+    int sh = 12;
+    while (((n + ((int64_t)1 << sh) - 1) >> sh) > RS_BLOCKS) ++sh;
+    return sh;
+}
+static_assert(RS_TILE == 1 << 12, "rs_shift starts at one tile");
+
+// The true count to the caller, the overflow condition, and the first pass's digit counts.
+__global__ void __launch_bounds__(RS_THREADS) hits_count_kernel(const unsigned long long *__restrict__ count,
+                                                                int64_t capacity, int64_t *__restrict__ count_out,
+                                                                uint32_t *__restrict__ status,
+                                                                const int64_t *__restrict__ hq,
+                                                                const int64_t *__restrict__ hr, int r_bits,
+                                                                uint32_t *__restrict__ table) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const unsigned long long c = *count;
+        *count_out = (int64_t)c;
+        if (c > (unsigned long long)capacity) atomicOr(status, ST_OVERFLOW);
     }
-}
-
-constexpr int SB = 2048;  // elements per shared-memory bitonic block
-
-// All passes j < SB/2.. of stage `size` (or every stage up to SB when
-// size == 0) inside blocks of SB contiguous elements.
-__global__ void __launch_bounds__(SB / 2) bitonic_smem_kernel(uint64_t *__restrict__ tmp, int64_t P,
-                                                              int64_t size) {
-    const uint64_t pn = tmp[1];
-    const int64_t base = (int64_t)blockIdx.x * SB;
-    if ((uint64_t)base >= pn) return;
-    if (size > 0 && (uint64_t)size > pn) return;
-    __shared__ uint64_t sk[SB];
-    __shared__ uint32_t sv[SB];
-    uint64_t *keys = tmp + 2;
-    uint32_t *vals = reinterpret_cast<uint32_t *>(tmp + 2 + P);
-    const int64_t live = ((int64_t)pn - base) < SB ? ((int64_t)pn - base) : SB;
-    for (int t = threadIdx.x; t < SB; t += blockDim.x) {
-        sk[t] = t < live ? keys[base + t] : KEY_EMPTY;
-        sv[t] = t < live ? vals[base + t] : 0u;
+    const int64_t n = hits_live(count, capacity);
+    const int sh = rs_shift(n);
+    const int64_t b0 = (int64_t)blockIdx.x << sh;
+    if (b0 >= n) return;
+    __shared__ uint32_t cnt[RS_DIGITS];
+    if (threadIdx.x < RS_DIGITS) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    for (int64_t i = b0 + threadIdx.x; i < min(n, b0 + ((int64_t)1 << sh)); i += RS_THREADS) {
+        const uint64_t key = ((uint64_t)hq[i] << r_bits) | (uint64_t)hr[i];
+        atomicAdd(&cnt[key & (RS_DIGITS - 1)], 1u);
     }
     __syncthreads();
-    auto pass = [&](int64_t sz, int j) {
-        for (int t = threadIdx.x; t < SB / 2; t += blockDim.x) {
-            int lo = 2 * t - (t & (j - 1));
-            int hi = lo + j;
-            int64_t gi = base + lo;
-            bool up = (gi & sz) == 0;
-            uint64_t a = sk[lo], b = sk[hi];
-            if ((a > b) == up) {
-                sk[lo] = b;
-                sk[hi] = a;
-                uint32_t tv = sv[lo];
-                sv[lo] = sv[hi];
-                sv[hi] = tv;
+    if (threadIdx.x < RS_DIGITS) table[(int64_t)blockIdx.x * RS_DIGITS + threadIdx.x] = cnt[threadIdx.x];
+}
+
+// One pass: digit (key >> shift) & 255.  FIRST reads the caller's (q, r,
+// score) triples, LAST writes them; passes between use keys and scores.
+// table: this pass's counts; next: the next pass's (zero before), unused
+// when LAST.
+template <bool FIRST, bool LAST>
+__global__ void __launch_bounds__(RS_THREADS)
+    hits_scatter_kernel(const unsigned long long *__restrict__ count, int64_t capacity, int r_bits, int shift,
+                        const uint32_t *__restrict__ table, uint32_t *__restrict__ next,
+                        const uint64_t *__restrict__ src_k, const int64_t *__restrict__ src_r,
+                        const uint32_t *__restrict__ src_v, uint64_t *__restrict__ dst_k, int64_t *__restrict__ dst_r,
+                        uint32_t *__restrict__ dst_v) {
+    const int64_t n = hits_live(count, capacity);
+    const int sh = rs_shift(n);
+    const int64_t b0 = (int64_t)blockIdx.x << sh, b1 = min(n, b0 + ((int64_t)1 << sh));
+    if (b0 >= n) return;
+    __shared__ uint16_t cnt[RS_WARPS][RS_DIGITS];  // of the tile, then each (warp, digit)'s first place in it
+    __shared__ uint64_t part[2][RS_GROUPS][RS_DIGITS];
+    __shared__ uint64_t place[RS_DIGITS];  // where this block's next element of a digit goes
+    __shared__ uint64_t wsum[RS_DIGITS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    {  // digit counts of every block, and of the blocks before this one
+        const int nb = (int)((n + ((int64_t)1 << sh) - 1) >> sh), d = tid % RS_DIGITS, g = tid / RS_DIGITS;
+        uint64_t tot = 0, pre = 0;
+#pragma unroll 8
+        for (int b = g; b < nb; b += RS_GROUPS) {
+            const uint32_t c = table[(int64_t)b * RS_DIGITS + d];
+            tot += c;
+            pre += b < (int)blockIdx.x ? c : 0u;
+        }
+        part[0][g][d] = tot;
+        part[1][g][d] = pre;
+    }
+    __syncthreads();
+    uint64_t before = 0, incl = 0;
+    if (tid < RS_DIGITS) {  // smaller digits anywhere, then this digit in earlier blocks
+        uint64_t t = 0;
+        for (int i = 0; i < RS_GROUPS; ++i) t += part[0][i][tid], before += part[1][i][tid];
+        incl = t;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint64_t x = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += x;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        before += incl - t;
+    }
+    __syncthreads();
+    if (tid < RS_DIGITS) {
+        for (int w = 0; w < warp; ++w) before += wsum[w];
+        place[tid] = before;
+    }
+    for (int64_t t0 = b0; t0 < b1; t0 += RS_TILE) {
+        // Elements in order: warp w takes 32 RS_ITEMS consecutive ones, 32 at a time.
+        uint64_t key[RS_ITEMS];
+        uint32_t val[RS_ITEMS], rank[RS_ITEMS];
+        const int64_t i0 = t0 + warp * (32 * RS_ITEMS) + lane;
+#pragma unroll
+        for (int it = 0; it < RS_ITEMS; ++it) {
+            const int64_t i = i0 + it * 32;
+            key[it] = 0;
+            val[it] = 0;
+            if (i < b1) {
+                key[it] = FIRST ? ((src_k[i] << r_bits) | (uint64_t)src_r[i]) : src_k[i];
+                val[it] = src_v[i];
+            }
+        }
+        for (int i = lane; i < RS_DIGITS; i += 32) cnt[warp][i] = 0;
+        __syncwarp();
+        // Rank within the warp: among equal digits, earlier elements first.
+#pragma unroll
+        for (int it = 0; it < RS_ITEMS; ++it) {
+            const bool live = i0 + it * 32 < b1;
+            const uint32_t dg = live ? (uint32_t)(key[it] >> shift) & (RS_DIGITS - 1) : RS_DIGITS;
+            const uint32_t peers = __match_any_sync(0xffffffffu, dg);
+            const uint32_t ahead = __popc(peers & ((1u << lane) - 1u));
+            const uint32_t seen = live ? cnt[warp][dg] : 0u;
+            __syncwarp();
+            if (live && ahead == 0) cnt[warp][dg] = (uint16_t)(seen + __popc(peers));
+            __syncwarp();
+            rank[it] = seen + ahead;
+        }
+        __syncthreads();
+        uint32_t in_tile = 0;  // this digit's elements in the tile
+        if (tid < RS_DIGITS) {
+#pragma unroll 8
+            for (int w = 0; w < RS_WARPS; ++w) {
+                const uint32_t c = cnt[w][tid];
+                cnt[w][tid] = (uint16_t)in_tile;
+                in_tile += c;
             }
         }
         __syncthreads();
-    };
-    if (size == 0) {
-        for (int64_t sz = 2; sz <= SB && (uint64_t)sz <= (pn > 1 ? pn : 2); sz <<= 1)
-            for (int j = (int)(sz >> 1); j > 0; j >>= 1) pass(sz, j);
-    } else {
-        for (int j = SB / 2; j > 0; j >>= 1) pass(size, j);
-    }
-    for (int t = threadIdx.x; t < live; t += blockDim.x) {
-        keys[base + t] = sk[t];
-        vals[base + t] = sv[t];
-    }
-}
-
-__global__ void bitonic_global_kernel(uint64_t *__restrict__ tmp, int64_t P, int64_t size, int64_t j) {
-    const uint64_t pn = tmp[1];
-    if ((uint64_t)size > pn) return;
-    uint64_t *keys = tmp + 2;
-    uint32_t *vals = reinterpret_cast<uint32_t *>(tmp + 2 + P);
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)pn / 2;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t lo = 2 * t - (t & (j - 1));
-        int64_t hi = lo + j;
-        bool up = (lo & size) == 0;
-        uint64_t a = keys[lo], b = keys[hi];
-        if ((a > b) == up) {
-            keys[lo] = b;
-            keys[hi] = a;
-            uint32_t tv = vals[lo];
-            vals[lo] = vals[hi];
-            vals[hi] = tv;
+#pragma unroll
+        for (int it = 0; it < RS_ITEMS; ++it) {
+            if (i0 + it * 32 >= b1) break;
+            const uint32_t dg = (uint32_t)(key[it] >> shift) & (RS_DIGITS - 1);
+            const uint64_t pos = place[dg] + cnt[warp][dg] + rank[it];
+            if (LAST) {
+                dst_k[pos] = key[it] >> r_bits;
+                dst_r[pos] = (int64_t)(key[it] & ((1ull << r_bits) - 1ull));
+            } else {
+                dst_k[pos] = key[it];
+                atomicAdd(&next[(int64_t)(pos >> sh) * RS_DIGITS +
+                                ((uint32_t)(key[it] >> (shift + RS_BITS)) & (RS_DIGITS - 1))],
+                          1u);
+            }
+            dst_v[pos] = val[it];
         }
+        __syncthreads();
+        if (tid < RS_DIGITS) place[tid] += in_tile;
     }
 }
 
-__global__ void hits_unpack_kernel(const uint64_t *__restrict__ tmp, int64_t P, int64_t *__restrict__ hq,
-                                   int64_t *__restrict__ hr, uint32_t *__restrict__ hs) {
-    const uint64_t n = tmp[0];
-    const uint64_t *keys = tmp + 2;
-    const uint32_t *vals = reinterpret_cast<const uint32_t *>(tmp + 2 + P);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; (uint64_t)i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        hq[i] = (int64_t)(keys[i] >> 32);
-        hr[i] = (int64_t)(uint32_t)keys[i];
-        hs[i] = vals[i];
-    }
+int bits_for(int64_t n) {  // bits of n - 1
+    int b = 0;
+    while (b < 62 && (1ll << b) < n) ++b;
+    return b;
 }
 
-int grid_for(int64_t n, int block) {
-    int64_t g = (n + block - 1) / block;
-    if (g > 4096) g = 4096;
-    return g < 1 ? 1 : (int)g;
-}
+int64_t hits_blocks(int64_t capacity) { return std::min<int64_t>(RS_BLOCKS, (capacity + RS_TILE - 1) / RS_TILE); }
 
 }  // namespace
 
-int64_t hits_sort_elems(int64_t capacity) {
-    int64_t p = 1;
-    while (p < capacity) p <<= 1;
-    return p < SB ? SB : p;
+int hits_passes(int64_t n_q, int64_t n_refs) {
+    const int bits = bits_for(n_q) + bits_for(n_refs);
+    return std::max(2, 2 * ((bits + 2 * RS_BITS - 1) / (2 * RS_BITS)));
+}
+
+HitsLayout hits_layout(int64_t capacity, int passes) {
+    HitsLayout L;
+    L.table = 256;  // the counter's line first
+    L.zero_bytes = L.table + (size_t)passes * hits_blocks(capacity) * RS_DIGITS * sizeof(uint32_t);
+    L.keys = (L.zero_bytes + 255) & ~size_t(255);
+    L.vals = L.keys + ((size_t)capacity * sizeof(uint64_t) + 255 & ~size_t(255));
+    L.bytes = L.vals + (size_t)capacity * sizeof(uint32_t);
+    return L;
 }
 
 // Warps per query for n_q queries of up to n lists: about MERGE_AHEAD lists a
@@ -430,22 +500,38 @@ cudaError_t launch_hits_block_offset(const unsigned long long *count, unsigned l
     return cudaGetLastError();
 }
 
-// sort_tmp must hold 2 + hits_sort_elems(capacity) * 1.5 u64 words.
-cudaError_t launch_hits_finish(unsigned long long *count, int64_t capacity, int64_t *hit_q,
-                               int64_t *hit_r, uint32_t *hit_score, int64_t *count_out,
-                               uint64_t *sort_tmp, uint32_t *status, cudaStream_t s) {
-    const int64_t P = hits_sort_elems(capacity);
-    hits_prep_kernel<<<1, 1, 0, s>>>(count, capacity, count_out, sort_tmp, status);
+cudaError_t launch_hits_finish(void *aux, int64_t capacity, int64_t n_q, int64_t n_refs, int64_t *hit_q,
+                               int64_t *hit_r, uint32_t *hit_score, int64_t *count_out, uint32_t *status,
+                               cudaStream_t s) {
+    const int passes = hits_passes(n_q, n_refs), r_bits = bits_for(n_refs);
+    const HitsLayout L = hits_layout(capacity, passes);
+    uint8_t *base = static_cast<uint8_t *>(aux);
+    const unsigned long long *count = reinterpret_cast<unsigned long long *>(base);
+    const int64_t nb = hits_blocks(capacity);
+    uint32_t *table = reinterpret_cast<uint32_t *>(base + L.table);
+    uint64_t *tk = reinterpret_cast<uint64_t *>(base + L.keys);
+    uint32_t *tv = reinterpret_cast<uint32_t *>(base + L.vals);
+    const unsigned grid = (unsigned)std::max<int64_t>(1, nb);
+    hits_count_kernel<<<grid, RS_THREADS, 0, s>>>(count, capacity, count_out, status, hit_q, hit_r, r_bits, table);
     if (capacity == 0) return cudaGetLastError();
-    hits_keys_kernel<<<grid_for(P, 256), 256, 0, s>>>(hit_q, hit_r, hit_score, sort_tmp, P);
-    const int nblk = (int)(P / SB);
-    bitonic_smem_kernel<<<nblk, SB / 2, 0, s>>>(sort_tmp, P, 0);
-    for (int64_t size = 2 * SB; size <= P; size <<= 1) {
-        for (int64_t j = size >> 1; j >= SB; j >>= 1)
-            bitonic_global_kernel<<<grid_for(P / 2, 256), 256, 0, s>>>(sort_tmp, P, size, j);
-        bitonic_smem_kernel<<<nblk, SB / 2, 0, s>>>(sort_tmp, P, size);
+    uint64_t *hk = reinterpret_cast<uint64_t *>(hit_q);
+    for (int p = 0; p < passes; ++p) {
+        const uint32_t *now = table + (int64_t)p * nb * RS_DIGITS;
+        uint32_t *next = table + (int64_t)(p + 1) * nb * RS_DIGITS;
+        const int shift = p * RS_BITS;
+        if (p == 0)
+            hits_scatter_kernel<true, false><<<grid, RS_THREADS, 0, s>>>(count, capacity, r_bits, shift, now, next, hk,
+                                                                         hit_r, hit_score, tk, nullptr, tv);
+        else if (p + 1 == passes)
+            hits_scatter_kernel<false, true><<<grid, RS_THREADS, 0, s>>>(count, capacity, r_bits, shift, now, nullptr,
+                                                                         tk, nullptr, tv, hk, hit_r, hit_score);
+        else if (p & 1)
+            hits_scatter_kernel<false, false><<<grid, RS_THREADS, 0, s>>>(count, capacity, r_bits, shift, now, next,
+                                                                          tk, nullptr, tv, hk, nullptr, hit_score);
+        else
+            hits_scatter_kernel<false, false><<<grid, RS_THREADS, 0, s>>>(count, capacity, r_bits, shift, now, next,
+                                                                          hk, nullptr, hit_score, tk, nullptr, tv);
     }
-    hits_unpack_kernel<<<grid_for(capacity, 256), 256, 0, s>>>(sort_tmp, P, hit_q, hit_r, hit_score);
     return cudaGetLastError();
 }
 

@@ -300,15 +300,15 @@ fastid_status fastid_compare_streamed(fastid_ctx *ctx, const uint64_t *refs_host
         }
     }
     unsigned long long *count = nullptr, *snaps = nullptr;
-    uint64_t *sort_tmp = nullptr;
+    const int passes = hits_passes(n_q, n_refs);
+    const HitsLayout HL = hits_layout(capacity, passes);
     auto setup = [&](StreamState &st) -> fastid_status {
         cudaError_t e = cudaSuccess;
-        uint8_t *aux = static_cast<uint8_t *>(st.take_extra(hits_aux_bytes(capacity), e));
+        uint8_t *aux = static_cast<uint8_t *>(st.take_extra(HL.bytes, e));
         snaps = static_cast<unsigned long long *>(st.take_extra((size_t)n_blocks * 8, e));
         if (e == cudaSuccess) {
             count = reinterpret_cast<unsigned long long *>(aux);
-            sort_tmp = reinterpret_cast<uint64_t *>(aux + 256);
-            e = cudaMemsetAsync(count, 0, sizeof(unsigned long long), s);
+            e = cudaMemsetAsync(aux, 0, HL.zero_bytes, s);
         }
         return e == cudaSuccess ? FASTID_OK : scuda(ctx, e, "hit counters");
     };
@@ -323,10 +323,10 @@ fastid_status fastid_compare_streamed(fastid_ctx *ctx, const uint64_t *refs_host
         return FASTID_OK;
     };
     if ((rs = stream_blocks(ctx, R, n_q, true, s, setup, compare)) != FASTID_OK) return rs;
-    cudaError_t e = launch_hits_finish(count, capacity, hit_q_dev, hit_r_dev, hit_score_dev, hit_count_dev, sort_tmp,
+    cudaError_t e = launch_hits_finish(count, capacity, n_q, n_refs, hit_q_dev, hit_r_dev, hit_score_dev, hit_count_dev,
                                        ctx->dev_status, s);
     if (e != cudaSuccess) return scuda(ctx, e, "hit list finish");
-    ctx->launches += hits_finish_launches(capacity);
+    ctx->launches += hits_finish_launches(capacity, passes);
     return FASTID_OK;
 }
 

@@ -438,16 +438,6 @@ struct TcSmem {
     int abort_flag;
 };
 
-__device__ __noinline__ void append_hit(unsigned long long *count, int64_t capacity, int64_t *hq, int64_t *hr,
-                                       uint32_t *hs, int64_t q, int64_t r, uint32_t sc) {
-    const unsigned long long pos = atomicAdd(count, 1ull);
-    if (pos < (unsigned long long)capacity) {
-        hq[pos] = q;
-        hr[pos] = r;
-        hs[pos] = sc;
-    }
-}
-
 // Writes a warp's 32 x 32 block of full-matrix scores (v: lane's operand row,
 // 32 columns) with rows of the output written whole.  Each lane storing its
 // own row touched 32 rows an instruction, 2 or 4 useful bytes of every
@@ -588,6 +578,33 @@ __device__ __forceinline__ GroupWork group_work(const TensorArgs &a, int64_t wg,
         w.slot = (int64_t)sc.slot0 + grid * cpg * sc.tpx + (t * cpg + rank) * sc.t_tpx;
     }
     return w;
+}
+
+// Appends a warp's hits in one 32-column block (m: lane's columns, taddr: the
+// block's TMEM address, references rch + j): one atomicAdd for the warp, then
+// the columns some lane needs, re-read from TMEM by the whole warp as in the
+// top-k path.
+__device__ __forceinline__ void append_hits(const TensorArgs &args, uint32_t m, uint32_t taddr, float cq, int64_t q,
+                                            int64_t rch, int lane) {
+    const uint32_t total = __reduce_add_sync(0xffffffffu, __popc(m));
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(args.hit_count, (unsigned long long)total);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    uint32_t mm = __reduce_or_sync(0xffffffffu, m);
+    while (mm != 0u) {
+        const int j = __ffs(mm) - 1;
+        mm &= mm - 1u;
+        const uint32_t d = tmem_ld1(taddr + j);
+        const bool hit = (m >> j) & 1u;
+        const uint32_t b = __ballot_sync(0xffffffffu, hit);
+        const unsigned long long pos = base + __popc(b & ((1u << lane) - 1u));
+        base += __popc(b);
+        if (hit && pos < (unsigned long long)args.capacity) {
+            args.hit_q[pos] = q;
+            args.hit_r[pos] = rch + j;
+            args.hit_score[pos] = (uint32_t)(int32_t)(__uint_as_float(d) + cq);
+        }
+    }
 }
 
 // Save / resume one thread's top-k list.  Slot layout [slot][k][128]: entry i
@@ -1092,12 +1109,7 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                             if (rch + 32 > n_refs) m &= rch >= n_refs ? 0u : ((1u << (n_refs - rch)) - 1u);
                             if (!__any_sync(0xffffffffu, m != 0u)) continue;
                             if (args.epi == EPI_HITS) {
-#pragma unroll
-                                for (int j = 0; j < 32; ++j)
-                                    if (m & (1u << j))
-                                        append_hit(args.hit_count, args.capacity, args.hit_q, args.hit_r,
-                                                   args.hit_score, q, rch + j,
-                                                   (uint32_t)(int32_t)(__uint_as_float(v[j]) + cq));
+                                append_hits(args, m, taddr + ch * 32, cq, q, rch, lane);
                                 continue;
                             }
                             // rare path: insert the candidates in lock-step, column by
