@@ -6,53 +6,96 @@ namespace fastid {
 
 namespace {
 
-// Four allele bytes -> four bits (byte i -> bit i).  Each byte is first
-// normalised to 0/1; the multiply then moves byte i (at bit 8i) to bit 24+i:
-// the multiplier 2^24 + 2^17 + 2^10 + 2^3 places byte i's term at 8i + 24 - 7j
-// for multiplier term j, so only i == j lands in bits 24..27, the i < j terms
-// land at distinct positions below bit 20 (no carries) and i > j overflow.
-__device__ __forceinline__ uint32_t bytes4_to_bits(uint32_t x) {
-    uint32_t nz = __vcmpne4(x, 0u) & 0x01010101u;
-    return (nz * 0x01020408u) >> 24;
+// Bit 7 of each byte of the result: that byte of x is not 0.
+__device__ __forceinline__ uint32_t nonzero4(uint32_t x) {
+    return (((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x) & 0x80808080u;
 }
 
-// One warp per row; lane handles 64-bit words lane, lane+32, ...
-__global__ void pack_kernel(const uint8_t *__restrict__ alleles, int64_t n, int32_t n_loci,
-                            int64_t ld_alleles, uint64_t *__restrict__ packed, int64_t ld_words,
-                            uint32_t *__restrict__ norms) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const bool vec = ((ld_alleles & 15) == 0) && ((reinterpret_cast<uintptr_t>(alleles) & 15) == 0);
-    for (int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < n;
-         row += warps_total) {
+// Eight allele bytes -> eight bits in the top byte.  Bytes of x go to bits 8i
+// and bytes of y to bits 8i + 4; the multiplier 2^24 + 2^17 + 2^10 + 2^3 moves
+// bit 8i to 24 + i and bit 8i + 4 to 28 + i by its term 2^(24 - 7i), the terms
+// j > i land at distinct positions below bit 24 (no carries) and j < i
+// overflow.
+__device__ __forceinline__ uint32_t bytes8_to_top(uint32_t x, uint32_t y) {
+    return ((nonzero4(x) >> 7) | (nonzero4(y) >> 3)) * 0x01020408u;
+}
+
+// Sixteen allele bytes -> 16 bits.
+__device__ __forceinline__ uint32_t bytes16_to_bits(const uint4 v) {
+    return __byte_perm(bytes8_to_top(v.x, v.y), bytes8_to_top(v.z, v.w), 0x4473) & 0xFFFFu;
+}
+
+// The word of `live` (1..64) loci at a, byte by byte.
+__device__ __noinline__ uint64_t word_bytewise(const uint8_t *a, int live) {
+    uint64_t word = 0;
+#pragma unroll 16
+    for (int t = 0; t < live; ++t) word |= (uint64_t)(a[t] != 0) << t;
+    return word;
+}
+
+// The same from the aligned 16-byte blocks that hold the loci, shifted into
+// place: all of the word's loads are in flight together, whatever its
+// alignment and length.  The blocks may reach into the next row or the gap
+// between rows, never outside the buffer's first to last allele [lo, hi).
+__device__ __forceinline__ uint64_t word_of(const uint8_t *a, int live, const uint8_t *lo, const uint8_t *hi) {
+    const uint32_t s = (uint32_t)(reinterpret_cast<uintptr_t>(a) & 15);
+    const uint8_t *p = a - s;
+    const int blocks = ((int)s + live + 15) >> 4;  // up to five
+    if (p < lo || p + 16 * blocks > hi) return word_bytewise(a, live);  // the buffer's first or last word
+    uint4 v[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) v[c] = c < blocks ? __ldg(reinterpret_cast<const uint4 *>(p) + c) : make_uint4(0, 0, 0, 0);
+    uint64_t word = (uint64_t)(bytes16_to_bits(v[0]) | (bytes16_to_bits(v[1]) << 16)) |
+                    ((uint64_t)(bytes16_to_bits(v[2]) | (bytes16_to_bits(v[3]) << 16)) << 32);
+    if (s) word = (word >> s) | ((uint64_t)bytes16_to_bits(v[4]) << (64 - s));
+    return live < 64 ? word & ((1ull << live) - 1ull) : word;
+}
+__device__ __noinline__ uint64_t word_of_call(const uint8_t *a, int live, const uint8_t *lo, const uint8_t *hi) {
+    return word_of(a, live, lo, hi);
+}
+
+// G = 1 << log_g lanes share a row and make its 64-bit words, one a lane and
+// step; without norms the words of a row are also spread over cpr groups.
+// ALIGNED: rows start on 16 bytes, so every word but a row's last is four
+// whole blocks.  HBM-bound at size; the register limits keep enough warps to
+// cover the loads (60 registers: 262,144 x 2048 at 101 us instead of 87), and
+// the conversion is 21 instructions for 16 bytes.  Against a warp a row with
+// words off 16 bytes and last words read byte by byte: 262,144 x 2047 890 ->
+// 105 us, 1M x 1000 1768 -> 205, 1M x 1024 273 -> 169, 2M x 200 1560 -> 95,
+// 1000 x 65,536 17.5 -> 12.5, 262,144 x 2048 88 -> 87 (6.9 TB/s).  Coalesced
+// blocks with four lanes a word and shuffles between them were slower (151 us).
+template <bool ALIGNED>
+__global__ void __launch_bounds__(256, ALIGNED ? 8 : 5)
+    pack_kernel(const uint8_t *__restrict__ alleles, int64_t n, int32_t n_loci, int64_t ld_alleles,
+                uint64_t *__restrict__ packed, int64_t ld_words, uint32_t *__restrict__ norms, int log_g,
+                int64_t cpr) {
+    const int g = 1 << log_g, lane = threadIdx.x & (g - 1);
+    const int64_t units = n * cpr, step = ((int64_t)gridDim.x * blockDim.x) >> log_g;
+    const uint8_t *lo = alleles, *hi = alleles + (n - 1) * ld_alleles + n_loci;
+    // (whole warps stay in the loop, for the norms' shuffles)
+    for (int64_t u0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) >> log_g; u0 < units; u0 += step) {
+        const int64_t u = u0 + ((threadIdx.x & 31) >> log_g);
+        const int64_t row = cpr == 1 ? u : u / cpr, part = cpr == 1 ? 0 : u - row * cpr;
         const uint8_t *a = alleles + row * ld_alleles;
-        uint64_t *o = packed + row * ld_words;
         uint32_t pc = 0;
-        for (int64_t w = lane; w < ld_words; w += 32) {
+        for (int64_t w = part * g + lane; u < units && w < ld_words; w += g * cpr) {
             uint64_t word = 0;
             const int64_t l0 = w * 64;
-            if (l0 + 64 <= n_loci && vec) {
+            if (ALIGNED && l0 + 64 <= n_loci) {
                 const uint4 *p = reinterpret_cast<const uint4 *>(a + l0);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint4 v = __ldg(p + c);
-                    uint64_t b = (uint64_t)bytes4_to_bits(v.x) | ((uint64_t)bytes4_to_bits(v.y) << 4) |
-                                 ((uint64_t)bytes4_to_bits(v.z) << 8) |
-                                 ((uint64_t)bytes4_to_bits(v.w) << 12);
-                    word |= b << (16 * c);
-                }
+                const uint4 v0 = __ldg(p), v1 = __ldg(p + 1), v2 = __ldg(p + 2), v3 = __ldg(p + 3);
+                word = (uint64_t)(bytes16_to_bits(v0) | (bytes16_to_bits(v1) << 16)) |
+                       ((uint64_t)(bytes16_to_bits(v2) | (bytes16_to_bits(v3) << 16)) << 32);
             } else if (l0 < n_loci) {
-                const int64_t lim = (n_loci - l0) < 64 ? (n_loci - l0) : 64;
-                for (int64_t t = 0; t < lim; ++t)
-                    word |= (uint64_t)(a[l0 + t] != 0) << t;
+                const int live = n_loci - l0 < 64 ? (int)(n_loci - l0) : 64;
+                word = ALIGNED ? word_of_call(a + l0, live, lo, hi) : word_of(a + l0, live, lo, hi);
             }
-            o[w] = word;
+            packed[row * ld_words + w] = word;
             pc += __popcll(word);
         }
         if (norms) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) pc += __shfl_xor_sync(0xffffffffu, pc, off);
-            if (lane == 0) norms[row] = pc;
+            for (int off = g >> 1; off > 0; off >>= 1) pc += __shfl_xor_sync(0xffffffffu, pc, off);
+            if (lane == 0 && u < units) norms[row] = pc;
         }
     }
 }
@@ -147,7 +190,17 @@ int warp_grid(int64_t rows, int warps_per_block) {
 cudaError_t launch_pack(const uint8_t *alleles, int64_t n, int32_t n_loci, int64_t ld_alleles,
                         uint64_t *packed, int64_t ld_words, uint32_t *norms, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    pack_kernel<<<warp_grid(n, 8), 256, 0, s>>>(alleles, n, n_loci, ld_alleles, packed, ld_words, norms);
+    // lanes a row: as many as it has words, up to a warp; more words than
+    // that go to further groups where no norm joins them
+    int log_g = 0;
+    while (log_g < 5 && (1 << log_g) < ld_words) ++log_g;
+    const int64_t cpr = norms ? 1 : (ld_words + (1 << log_g) - 1) >> log_g;
+    const bool aligned = ((ld_alleles | (int64_t)reinterpret_cast<uintptr_t>(alleles)) & 15) == 0;
+    const int grid = warp_grid(((n * cpr << log_g) + 31) >> 5, 8);
+    if (aligned)
+        pack_kernel<true><<<grid, 256, 0, s>>>(alleles, n, n_loci, ld_alleles, packed, ld_words, norms, log_g, cpr);
+    else
+        pack_kernel<false><<<grid, 256, 0, s>>>(alleles, n, n_loci, ld_alleles, packed, ld_words, norms, log_g, cpr);
     return cudaGetLastError();
 }
 
