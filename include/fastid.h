@@ -299,16 +299,18 @@ fastid_status fastid_compare(fastid_ctx *ctx, const fastid_refdb *db, const uint
  *              and unchanged until the stream has passed this call.
  *  n_refs      1 .. 2^31 - 1;  flags: 0 or FASTID_REFS_TENSOR (expand each
  *              block to the FP8 operand, which FASTID_FORM_TENSOR then reads).
- *              Every other case reads each block's packed rows in the
- *              context's form: plain, or FP8 or FP4 expanded on chip
- *              (FASTID_FORM_AUTO: FP4).
+ *              Every other case reads each block in the context's form: plain,
+ *              FP8 expanded on chip, or FP4 (also FASTID_FORM_AUTO) -- for more
+ *              than 128 queries through an FP4 operand built per block where
+ *              the device has the memory, else expanded on chip.
  *  block_refs  largest block (>= 1; the first blocks are smaller, from
  *              block_refs / 8 doubling, so that the first comparison starts
  *              early).  Two blocks are on the device at once, each holding
  *              ceil(n_loci / 64) x 8 bytes per reference as copied plus, for
  *              the tensor form, its FP8 operand (n_loci rounded up to 128
- *              bytes per reference) or, for the plain form, padded rows and
- *              popcounts.
+ *              bytes per reference) or FP4 operand (n_loci rounded up to 256,
+ *              half a byte each) or, for the plain form and forms expanded on
+ *              chip, padded rows and popcounts.
  *  The other arguments are those of fastid_topk.  Stream-ordered: the call
  *  enqueues the copies and kernels and returns without waiting for them.
  * Errors: EINVAL, ENOMEM, ECUDA.

@@ -4,12 +4,13 @@
 // comparison and the k-lists folded on the device.
 //
 // Two slots, each a device staging buffer (the block as copied, host row
-// stride dropped) and a block database (padded rows + norms, and the FP8
-// operand with its TMA maps).  Block b uses slot s = b % 2 on three streams:
+// stride dropped) and a block database (padded rows + norms, or the FP8 or FP4
+// operand, with the TMA maps).  Block b uses slot s = b % 2 on three streams:
 //   copy:    wait expanded[s] (block b - 2 done with staging) -> H2D copy into
 //            staging[s] -> record copied[s]
 //   expand:  wait copied[s], compared[s] (block b - 2 done with the database)
-//            -> rows + norms (+ FP8 operand) of db[s] -> record expanded[s]
+//            -> rows + norms, or the FP8 or FP4 operand, of db[s] -> record
+//            expanded[s]
 //   compute: wait expanded[s] -> top-k of db[s] -> fold -> record compared[s]
 // so block b + 1's copy and expansion, and block b + 2's copy, run while
 // block b is compared.  Block sizes ramp up from an eighth of block_refs so
@@ -95,6 +96,7 @@ struct StreamState {
             if (sl.db.packed) cudaFreeAsync(sl.db.packed, s);
             if (sl.db.norms) cudaFreeAsync(sl.db.norms, s);
             if (sl.db.fp8) cudaFreeAsync(sl.db.fp8, s);
+            if (sl.db.fp4) cudaFreeAsync(sl.db.fp4, s);
         }
         for (void *p : extra) cudaFreeAsync(p, s);
         cudaEvent_t evs[] = {ready, copied[0], copied[1], expanded[0], expanded[1],
@@ -126,26 +128,52 @@ fastid_status check_refs(fastid_ctx *ctx, const StreamRefs &r) {
     return FASTID_OK;
 }
 
+// Both slots' FP4 operands.  They take up to four times the packed rows'
+// memory, so where they do not fit -- or would leave too little for the
+// comparisons' own scratch (query operand and top-k lists), which is taken
+// and given back here to see -- the call goes on over packed rows: false,
+// nothing held.
+bool take_fp4(StreamState &st, int64_t cap, int64_t n_q, int32_t k) {
+    cudaError_t e = cudaSuccess;
+    const size_t kb = (size_t)st.slot[0].db.kbytes4;
+    for (Slot &sl : st.slot) sl.db.fp4 = static_cast<uint8_t *>(st.take((size_t)cap * kb, e));
+    const size_t tiles = (size_t)rup(n_q, 2 * TC_TILE_Q) / TC_TILE_Q;
+    void *probe = st.take(tiles * TC_TILE_Q * (kb + 4) + (4 * (size_t)st.ctx->grid_tensor + 4 * tiles) * TC_TILE_Q * k * 8,
+                          e);
+    if (probe) cudaFreeAsync(probe, st.s);
+    if (e == cudaSuccess) return true;
+    cudaGetLastError();
+    for (Slot &sl : st.slot) {
+        if (sl.db.fp4) cudaFreeAsync(sl.db.fp4, st.s);
+        sl.db.fp4 = nullptr;
+    }
+    return false;
+}
+
 // The block pipeline (see the top of this file).  `setup(st)` allocates the
 // entry point's own buffers (take_extra) and enqueues its initial work on the
 // caller's stream; `compare(b, db, r0)` enqueues block b's comparison of
 // db (references r0 .. r0 + db.n_refs - 1) there.
 template <class Setup, class Compare>
-fastid_status stream_blocks(fastid_ctx *ctx, const StreamRefs &R, int64_t n_q, bool slots16, cudaStream_t s,
-                            Setup setup, Compare compare) {
+fastid_status stream_blocks(fastid_ctx *ctx, const StreamRefs &R, int64_t n_q, int32_t k, cudaStream_t s, Setup setup,
+                            Compare compare) {
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return scuda(ctx, e, "cudaSetDevice");
     const int32_t n_words = (R.n_loci + 63) / 64;
     const int64_t block = std::min<int64_t>(R.block_refs, R.n_refs);
     const int64_t cap = rup(block, ROW_ALIGN);
     // The operand the per-block comparisons will take (as the comparison
-    // calls pick it): the FP8 operand is built per block only for the tensor
-    // form over the FP8 copy; the plain form and the tensor form over packed
-    // rows read the padded rows.
-    // An FP4 form takes the packed rows of each block, expanded on chip.
-    const int op = pick_operand(ctx->form, (R.flags & FASTID_REFS_TENSOR) != 0, false, n_q, slots16);
+    // calls pick it from what the block database holds): the FP8 operand only
+    // for the tensor form over the FP8 copy; in an FP4 form the FP4 operand
+    // for more than one query tile, where the comparison over it is up to
+    // twice as fast as over packed rows expanded on chip and building it (32
+    // loci to 16 bytes, at the HBM rate) hides behind the previous block;
+    // else the padded rows.  (2048 queries x 4M at N = 2048, k = 32, blocks of
+    // 1M: 11.3 ms over packed rows, 9.5 over the operand.)
+    const int op = pick_operand(ctx->form, (R.flags & FASTID_REFS_TENSOR) != 0, n_q > AUTO_FP4_PACKED_MAX_Q, n_q,
+                                k <= 16);
     const bool tensor = op == OP_FP8;
-    const bool rows = !tensor;
+    bool f4 = op == OP_FP4;
 
     StreamState st(ctx, s);
     if ((e = st.init()) != cudaSuccess) return scuda(ctx, e, "streams and events");
@@ -162,6 +190,18 @@ fastid_status stream_blocks(fastid_ctx *ctx, const StreamRefs &R, int64_t n_q, b
         db.kpad = kpad;
         db.kbytes4 = tensor_kbytes4(R.n_loci);
         sl.staging = static_cast<uint64_t *>(st.take((size_t)block * n_words * 8, e));
+    }
+    if (e != cudaSuccess) return scuda(ctx, e, "block buffers");
+    fastid_status rs = setup(st);
+    if (rs != FASTID_OK) return rs;
+    if (f4) f4 = take_fp4(st, cap, n_q, k);
+    const bool rows = !tensor && !f4;
+    for (Slot &sl : st.slot) {
+        fastid_refdb &db = sl.db;
+        if (f4) {
+            if (e == cudaSuccess) e = make_operand_map(&db.map_b4, db.fp4, cap, db.kbytes4, tensor_tile_r4());
+            if (e == cudaSuccess) e = make_operand_map(&db.map_b4_half, db.fp4, cap, db.kbytes4, tensor_tile_r4() / 2);
+        }
         if (rows) {
             db.packed = static_cast<uint64_t *>(st.take((size_t)cap * ld64 * 8, e));
             db.norms = static_cast<uint32_t *>(st.take((size_t)cap * 4, e));
@@ -175,8 +215,6 @@ fastid_status stream_blocks(fastid_ctx *ctx, const StreamRefs &R, int64_t n_q, b
         }
     }
     if (e != cudaSuccess) return scuda(ctx, e, "block buffers");
-    fastid_status rs = setup(st);
-    if (rs != FASTID_OK) return rs;
     // the side streams may touch the pool allocations only after they exist
     if ((e = cudaEventRecord(st.ready, s)) != cudaSuccess || (e = cudaStreamWaitEvent(st.copy, st.ready, 0)) ||
         (e = cudaStreamWaitEvent(st.expand, st.ready, 0)))
@@ -204,11 +242,16 @@ fastid_status stream_blocks(fastid_ctx *ctx, const StreamRefs &R, int64_t n_q, b
             e = launch_copy_rows(sl.staging, n, n_words, n_words, db.packed, db.n_pad, ld64, db.norms, st.expand);
             ctx->launches += 1;
         }
-        // The FP8 operand straight from the staged rows, on a full grid: it
+        // The FP8 or FP4 operand straight from the staged rows, on a full grid: it
         // runs beside the previous block's comparison, and the sooner it is
         // done the less it slows it down.
         if (e == cudaSuccess && tensor) {
             e = launch_refs_e4m3(sl.staging, n_words, n, n_words, db.n_pad, kpad, db.fp8, ctx->grid_tensor * 32,
+                                 st.expand);
+            ctx->launches += 1;
+        }
+        if (e == cudaSuccess && f4) {
+            e = launch_refs_e2m1(sl.staging, n_words, n, n_words, db.n_pad, db.kbytes4, db.fp4, ctx->grid_tensor * 32,
                                  st.expand);
             ctx->launches += 1;
         }
@@ -263,7 +306,7 @@ fastid_status fastid_topk_streamed(fastid_ctx *ctx, const uint64_t *refs_host, i
         ctx->launches += 1;
         return FASTID_OK;
     };
-    return stream_blocks(ctx, R, n_q, k <= 16, s, setup, compare);
+    return stream_blocks(ctx, R, n_q, k, s, setup, compare);
 }
 
 fastid_status fastid_compare_streamed(fastid_ctx *ctx, const uint64_t *refs_host, int64_t n_refs, int32_t n_loci,
@@ -322,7 +365,7 @@ fastid_status fastid_compare_streamed(fastid_ctx *ctx, const uint64_t *refs_host
         ctx->launches += r0 != 0 && capacity > 0 ? 2 : 1;
         return FASTID_OK;
     };
-    if ((rs = stream_blocks(ctx, R, n_q, true, s, setup, compare)) != FASTID_OK) return rs;
+    if ((rs = stream_blocks(ctx, R, n_q, 1, s, setup, compare)) != FASTID_OK) return rs;
     cudaError_t e = launch_hits_finish(count, capacity, n_q, n_refs, hit_q_dev, hit_r_dev, hit_score_dev, hit_count_dev,
                                        ctx->dev_status, s);
     if (e != cudaSuccess) return scuda(ctx, e, "hit list finish");
