@@ -85,6 +85,10 @@ struct TcShape {
     static constexpr int STAGES = RING - (SC && (BN == 224) != PK ? 1 : 0);
     static constexpr uint32_t B_BYTES = (uint32_t)(CG2 ? BN / 2 : BN) * TC_BK;
     static constexpr uint32_t TMEM_COLS = BN == 128 ? 256 : 512;
+    // beside the ring: transpose buffers, or the candidate queues (QD entries
+    // a query row: 8, or what the fullest ring leaves)
+    static constexpr int QD = CG2 && BN == 256 ? 3 : 8;
+    static constexpr uint32_t EX_BYTES = SC ? SC_BYTES : (uint32_t)QD * TC_BM * 4;
 };
 
 // One database ("panel") of a launch, with its schedule (TcSched).
@@ -427,6 +431,37 @@ __device__ __forceinline__ void net_insert(int32_t (&ls)[KM], uint32_t (&lr)[KM]
     lr[0] = first ? xr : lr[0];
 }
 
+// Candidate queues.  A candidate (a score that beats its query's current
+// cut) goes to its query's queue in shared memory -- score in the high bits,
+// reference relative to a window of TC_QSPAN in the low ones -- and the 32
+// lanes of a warp insert their queues together when one of them is full.
+// Inserting each candidate on arrival ran the 80 to 160 instructions of
+// net_insert for one lane's candidate while the other 31 had none: with short
+// streams, whose lists are still filling, that took most of a launch (a block
+// of 131,072 references against 2048 queries, k = 32: 737 us, of which the
+// MMAs are 107).  Entries leave in arrival order, so equal scores still keep
+// the lower reference first; one that no longer beats the list changes
+// nothing.  The cut is that of the last insertion, so a deeper queue lets more
+// late candidates in: with k = 16 and 8 entries about a fifth more.
+constexpr int TC_QBITS = 15;  // 17 bits hold any score (N <= 65536)
+constexpr int64_t TC_QSPAN = 1ll << TC_QBITS;
+
+template <int KM>
+__device__ __forceinline__ void queue_insert(const uint32_t *queue, int queued, int64_t qbase, int32_t (&ls)[KM],
+                                             uint32_t (&lr)[KM]) {
+    const int n = (int)__reduce_max_sync(0xffffffffu, (uint32_t)queued);
+    for (int i = 0; i < n; ++i) {
+        int32_t xs = NET_EMPTY;
+        uint32_t xr = 0u;
+        if (i < queued) {
+            const uint32_t e = queue[i * TC_BM];
+            xs = (int32_t)(e >> TC_QBITS);
+            xr = (uint32_t)qbase + (e & (uint32_t)(TC_QSPAN - 1));
+        }
+        if (__any_sync(0xffffffffu, xs < ls[KM - 1])) net_insert(ls, lr, xs, xr);
+    }
+}
+
 struct TcSmem {
     uint64_t full[8];
     uint64_t empty[8];
@@ -749,8 +784,8 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
     uint8_t *sA = base;
     uint8_t *sB = base + S::STAGES * TC_A_BYTES;
     uint8_t *sP = base + S::STAGES * (TC_A_BYTES + S::B_BYTES);  // PK only
-    uint8_t *sT = sP + (PK ? S::STAGES * P_BYTES : 0);  // SC only
-    TcSmem *ctl = reinterpret_cast<TcSmem *>(sT + (SC ? SC_BYTES : 0));
+    uint8_t *sT = sP + (PK ? S::STAGES * P_BYTES : 0);  // transpose buffers or candidate queues
+    TcSmem *ctl = reinterpret_cast<TcSmem *>(sT + S::EX_BYTES);
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -1066,6 +1101,14 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                         }
                     }
                     float cut = ls[KM - 1] == NET_EMPTY ? cut0 : (float)ls[KM - 1] - cq;
+                    uint32_t *queue = reinterpret_cast<uint32_t *>(sT) + row;  // entry i at i * TC_BM (see queue_insert)
+                    int queued = 0;
+                    int64_t qbase = rc * BN;
+                    auto flush = [&]() {
+                        queue_insert(queue, queued, qbase, ls, lr);
+                        queued = 0;
+                        cut = ls[KM - 1] == NET_EMPTY ? cut0 : (float)ls[KM - 1] - cq;
+                    };
                     for (int64_t rt = rc; rt < re; ++rt) {
                         const bool got = mbar_wait(smem_u32(&ctl->tfull[acc]), acc_phase, abort_flag, args.status, 6);
                         __syncwarp();
@@ -1075,6 +1118,10 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                         }
                         tc_fence_after();
                         const int64_t r0 = rt * BN;
+                        if (topk && r0 + BN - qbase > TC_QSPAN) {  // the queues' reference window moves on
+                            flush();
+                            qbase = r0;
+                        }
                         const uint32_t taddr = tmem_base + lane_addr + (uint32_t)(acc * BN);
 #pragma unroll 1
                         for (int ch = 0; ch < BN / 32; ++ch) {
@@ -1112,24 +1159,49 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                                 append_hits(args, m, taddr + ch * 32, cq, q, rch, lane);
                                 continue;
                             }
-                            // rare path: insert the candidates in lock-step, column by
-                            // column in increasing order (so each lane inserts its own
-                            // in increasing reference order); a column some lane needs
-                            // is re-read from TMEM by the whole warp (the accumulator
-                            // is released only after the tile, below)
-                            uint32_t mm = __reduce_or_sync(0xffffffffu, m);
-                            while (mm != 0u) {
-                                const int j = __ffs(mm) - 1;
-                                mm &= mm - 1u;
-                                const float d = __uint_as_float(tmem_ld1(taddr + ch * 32 + j));
-                                int32_t xs = NET_EMPTY;
-                                uint32_t xr = 0u;
-                                if (((m >> j) & 1u) && d < cut) {
-                                    xs = (int32_t)(d + cq);
-                                    xr = (uint32_t)(rch + j);
+                            // rare path.  The candidates go to the queues; where they do
+                            // not fit, the queues are inserted first, and a chunk that
+                            // is dense even then (a list still filling) is inserted
+                            // directly, in lock-step and column by column, each column
+                            // re-read from TMEM by the whole warp (the accumulator is
+                            // released only after the tile, below).
+                            if (__any_sync(0xffffffffu, queued + __popc(m) > S::QD)) {
+                                flush();
+                                uint32_t still = 0;
+#pragma unroll
+                                for (int j = 0; j < 32; ++j) still |= (uint32_t)(__uint_as_float(v[j]) < cut) << j;
+                                m &= still;
+                                if (__any_sync(0xffffffffu, __popc(m) > S::QD)) {
+                                    uint32_t mm = __reduce_or_sync(0xffffffffu, m);
+                                    while (mm != 0u) {
+                                        const int j = __ffs(mm) - 1;
+                                        mm &= mm - 1u;
+                                        const float d = __uint_as_float(tmem_ld1(taddr + ch * 32 + j));
+                                        int32_t xs = NET_EMPTY;
+                                        uint32_t xr = 0u;
+                                        if (((m >> j) & 1u) && d < cut) {
+                                            xs = (int32_t)(d + cq);
+                                            xr = (uint32_t)(rch + j);
+                                        }
+                                        net_insert(ls, lr, xs, xr);
+                                        cut = ls[KM - 1] == NET_EMPTY ? cut0 : (float)ls[KM - 1] - cq;
+                                    }
+                                    continue;
                                 }
-                                net_insert(ls, lr, xs, xr);
-                                cut = ls[KM - 1] == NET_EMPTY ? cut0 : (float)ls[KM - 1] - cq;
+                            }
+                            const uint32_t mm = __reduce_or_sync(0xffffffffu, m);
+                            const uint32_t rel = (uint32_t)(rch - qbase);
+#pragma unroll
+                            for (int g = 0; g < 32; g += 8) {
+                                if (((mm >> g) & 0xFFu) == 0u) continue;
+#pragma unroll
+                                for (int j = g; j < g + 8; ++j) {
+                                    if ((m >> j) & 1u) {
+                                        queue[queued * TC_BM] =
+                                            ((uint32_t)(int32_t)(__uint_as_float(v[j]) + cq) << TC_QBITS) | (rel + j);
+                                        ++queued;
+                                    }
+                                }
                             }
                         }
                         // every column of the tile is processed: the MMA may reuse the accumulator
@@ -1143,7 +1215,10 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                             acc_phase ^= 1u;
                         }
                     }
-                    if (topk && ok) list_save(slot, ls, lr, k);
+                    if (topk && ok) {
+                        flush();
+                        list_save(slot, ls, lr, k);
+                    }
                 }
             }
         }
@@ -1357,7 +1432,7 @@ template <int BN, bool PK = false, bool CG2 = false, bool SC = false>
 size_t tensor_smem(bool f4 = false) {
     using S = TcShape<BN, PK, CG2, SC>;
     return 1024 + S::STAGES * (size_t)(TC_A_BYTES + S::B_BYTES + (PK ? pk_stage_bytes(BN, f4) : 0)) +
-           (SC ? SC_BYTES : 0) + 256;
+           S::EX_BYTES + 256;
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link
