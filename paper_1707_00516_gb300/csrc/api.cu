@@ -516,12 +516,14 @@ struct TensorPrep {
 
 enum ExtraKind { EXTRA_NONE, EXTRA_TOPK };
 
+// run_s, run_i: running lists whose k-th scores start the shared cuts, or NULL.
 // op (an operand other than OP_PLAIN): FP8 or FP4 operands; packed rows
 // expanded on chip are unpaired, and their FP8 queries are encoded at half
 // scale to match the expanded 2.0.
 fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint64_t *q, int64_t ld_q, int64_t n_q,
                              const uint8_t *modes, cudaStream_t s, Scratch &scr, ExtraKind ek, int64_t karg,
-                             size_t *extra_off, TensorPrep *tp, int op) {
+                             size_t *extra_off, TensorPrep *tp, int op, const uint32_t *run_s = nullptr,
+                             const int64_t *run_i = nullptr) {
     TcLaunch &L = tp->L;
     memset(&L, 0, sizeof L);
     const bool pk = op_packed(op), f4 = op_f4(op);
@@ -548,8 +550,10 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
     Carver cv;
     size_t o_a = cv.take<uint8_t>((size_t)n_q_pad * kbytes);
     size_t o_c = cv.take<float>((size_t)n_q_pad);
+    size_t o_g = cv.take<int32_t>(ek == EXTRA_TOPK ? (size_t)n_q_pad : 0);
     *extra_off = cv.take<uint8_t>(extra);
     FASTID_CUDA(ctx, scr.alloc(cv.off));
+    const SharedCut cut{ek == EXTRA_TOPK ? at<int32_t>(scr.p, o_g) : nullptr, run_s, run_i, (int32_t)karg};
     uint8_t *a = at<uint8_t>(scr.p, o_a);
     float *qconst = at<float>(scr.p, o_c);
     // spread the input queries over every tile of the operand (see
@@ -557,10 +561,10 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
     const int64_t spread = n_q_pad / tensor_tile_q();
     if (f4)
         FASTID_CUDA(ctx, launch_queries_e2m1(q, ld_q, n_q, db->n_words64, db->n_loci, modes, n_q_pad, kbytes, a,
-                                             qconst, spread, s));
+                                             qconst, spread, cut, s));
     else
         FASTID_CUDA(ctx, launch_queries_e4m3(q, ld_q, n_q, db->n_words64, db->n_loci, modes, n_q_pad, kbytes, a,
-                                             qconst, pk, spread, s));
+                                             qconst, pk, spread, cut, s));
     count_launches(ctx, 1);
     FASTID_CUDA(ctx, make_operand_map(&L.map_a[0], a, n_q_pad, kbytes, tensor_tile_q()));
     L.n_panels = 1;
@@ -573,6 +577,7 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
     L.n_rt[0] = n_rt;
     L.kpad[0] = kbytes;
     L.qconst[0] = qconst;
+    L.gcut[0] = cut.out;
     L.qspread[0] = (int32_t)spread;
     L.status = ctx->dev_status;
     return FASTID_OK;
@@ -700,7 +705,8 @@ fastid_status fastid_topk_accumulate(fastid_ctx *ctx, const fastid_refdb *db, in
     if (op) {
         TensorPrep tp;
         size_t xo;
-        if ((st = prepare_tensor(ctx, db, queries_dev, ld_q, n_q, modes_dev, s, scr, EXTRA_TOPK, k, &xo, &tp, op)))
+        if ((st = prepare_tensor(ctx, db, queries_dev, ld_q, n_q, modes_dev, s, scr, EXTRA_TOPK, k, &xo, &tp, op,
+                                 run_scores_dev, run_idx_dev)))
             return st;
         uint64_t *partial = at<uint64_t>(scr.p, xo);
         tp.L.epi = EPI_TOPK;

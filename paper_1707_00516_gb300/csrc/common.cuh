@@ -74,6 +74,7 @@ struct PrepJob {
     const uint8_t *mode;   // its mode byte
     uint8_t *dst;          // operand row [kpad bytes]: e4m3, or e2m1 when f4
     float *qc;             // its c_q
+    int32_t *gc;           // its shared cut (see TcLaunch::gcut)
     int32_t n_words;
     int32_t n_loci;
     int32_t kpad;          // operand row bytes
@@ -149,6 +150,12 @@ struct TcLaunch {
     int64_t n_rt[TC_MAXP];
     int32_t kpad[TC_MAXP];  // operand row bytes (a multiple of 128)
     const float *qconst[TC_MAXP];
+    // EPI_TOPK: one score per operand row that no result entry of the query
+    // exceeds, shared by every slice of the launch and lowered by each as its
+    // list fills (set by the encoders to none, or to a running list's k-th).
+    // Candidates of a higher score are dropped, those of the same score are not
+    // (their reference may be lower).
+    int32_t *gcut[TC_MAXP];
     // Query spreading (see spread_row_to_query): the panel's operand tiles
     // (0 or 1: operand row r holds input query r).  Batched plans spread each
     // panel's queries in batch order and give the merge their rows.
@@ -237,13 +244,22 @@ int tensor_tile_r();
 int tensor_kpad(int32_t n_loci);
 int tensor_grid_target(int device);
 int tensor_pair_clusters(int device);
+// Initial shared cuts (TcLaunch::gcut) written by the query encoders: per
+// operand row, into out (nullptr: none), the k-th score of the query's running
+// list where that list is full.
+struct SharedCut {
+    int32_t *out;
+    const uint32_t *run_s;  // [n_q][k], or nullptr
+    const int64_t *run_i;
+    int32_t k;
+};
 // FP8 reference operand [n_rows][kpad] from packed rows (n_src rows of n_words
 // words exist at stride ld64; zero elsewhere), on at most max_blocks CTAs.
 cudaError_t launch_refs_e4m3(const uint64_t *packed, int64_t ld64, int64_t n_src, int32_t n_words, int64_t n_rows,
                              int32_t kpad, uint8_t *out, int max_blocks, cudaStream_t s);
 cudaError_t launch_queries_e4m3(const uint64_t *q, int64_t ld_q, int64_t n_q, int32_t n_words, int32_t n_loci,
                                 const uint8_t *modes, int64_t n_q_pad, int32_t kpad, uint8_t *out, float *qconst,
-                                bool half, int64_t spread, cudaStream_t s);
+                                bool half, int64_t spread, const SharedCut &cut, cudaStream_t s);
 // TMA map over packed rows for packed-reference (PK) launches: boxes of 2
 // words x 256 rows (FP8 stages) or 4 words x 224 rows (FP4 stages).
 cudaError_t make_packed_map(CUtensorMap *map, const uint64_t *packed, int64_t rows, int64_t ld64, int box_words = 2,
@@ -256,7 +272,7 @@ cudaError_t launch_refs_e2m1(const uint64_t *packed, int64_t ld64, int64_t n_src
                              int32_t kbytes, uint8_t *out, int max_blocks, cudaStream_t s);
 cudaError_t launch_queries_e2m1(const uint64_t *q, int64_t ld_q, int64_t n_q, int32_t n_words, int32_t n_loci,
                                 const uint8_t *modes, int64_t n_q_pad, int32_t kbytes, uint8_t *out, float *qconst,
-                                int64_t spread, cudaStream_t s);
+                                int64_t spread, const SharedCut &cut, cudaStream_t s);
 
 cudaError_t launch_tensor_multi(int bn, const TcLaunch &L, cudaStream_t s);
 cudaError_t launch_prep_jobs(const PrepJob *jobs, int64_t n_jobs, cudaStream_t s);

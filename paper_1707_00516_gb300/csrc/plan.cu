@@ -167,11 +167,12 @@ fastid_status fastid_plan_create(fastid_ctx *ctx, const fastid_refdb *const *dbs
         off += bytes;
         return at;
     };
-    std::vector<size_t> o_a(n_panels), o_qc(n_panels);
+    std::vector<size_t> o_a(n_panels), o_qc(n_panels), o_gc(n_panels);
     int64_t n_prep = 0;
     for (int p = 0; p < n_panels; ++p) {
         o_a[p] = take((size_t)rows_pad[p] * kbytes(p));
         o_qc[p] = take((size_t)rows_pad[p] * sizeof(float));
+        o_gc[p] = take((size_t)rows_pad[p] * sizeof(int32_t));
         n_prep += rows_pad[p];
     }
     const size_t o_prep = take((size_t)n_prep * sizeof(PrepJob));
@@ -205,6 +206,7 @@ fastid_status fastid_plan_create(fastid_ctx *ctx, const fastid_refdb *const *dbs
                 j.mode = nullptr;
                 j.dst = W + o_a[p] + (size_t)r * kbytes(p);
                 j.qc = reinterpret_cast<float *>(W + o_qc[p]) + r;
+                j.gc = reinterpret_cast<int32_t *>(W + o_gc[p]) + r;
                 j.n_words = dbs[p]->n_words64;
                 j.n_loci = dbs[p]->n_loci;
                 j.kpad = (int32_t)kbytes(p);
@@ -254,6 +256,7 @@ fastid_status fastid_plan_create(fastid_ctx *ctx, const fastid_refdb *const *dbs
         L.n_rt[p] = n_rt[p];
         L.kpad[p] = (int32_t)kbytes(p);
         L.qconst[p] = reinterpret_cast<const float *>(W + o_qc[p]);
+        L.gcut[p] = reinterpret_cast<int32_t *>(W + o_gc[p]);
         L.qspread[p] = (int32_t)(rows_pad[p] / TC_TILE_Q);  // see the prep jobs
     }
     L.k = k;

@@ -1,7 +1,7 @@
 // fastid_topk_streamed: top-k over host-resident references, copied to the
 // device block by block (the blocked transfer of the known profiles in
 // Sec. III-C), with each block's loading overlapping the previous block's
-// comparison and the k-lists folded on the device.
+// comparison and the k-lists merged on the device.
 //
 // Two slots, each a device staging buffer (the block as copied, host row
 // stride dropped) and a block database (padded rows + norms, or the FP8 or FP4
@@ -11,7 +11,7 @@
 //   expand:  wait copied[s], compared[s] (block b - 2 done with the database)
 //            -> rows + norms, or the FP8 or FP4 operand, of db[s] -> record
 //            expanded[s]
-//   compute: wait expanded[s] -> top-k of db[s] -> fold -> record compared[s]
+//   compute: wait expanded[s] -> top-k of db[s] merged into the result -> record compared[s]
 // so block b + 1's copy and expansion, and block b + 2's copy, run while
 // block b is compared.  Block sizes ramp up from an eighth of block_refs so
 // that little loading is exposed before the first comparison.  All device
@@ -287,24 +287,15 @@ fastid_status fastid_topk_streamed(fastid_ctx *ctx, const uint64_t *refs_host, i
     if (n_q > 0 && (!out_scores_dev || !out_idx_dev)) return sfail(ctx, FASTID_EINVAL, "output is NULL");
     if (n_q == 0) return FASTID_OK;
     const cudaStream_t s = (cudaStream_t)stream;
-    uint32_t *blk_s = nullptr;  // one block's lists [n_q][k]
-    int64_t *blk_i = nullptr;
-    auto setup = [&](StreamState &st) -> fastid_status {
-        cudaError_t e = cudaSuccess;
-        blk_s = static_cast<uint32_t *>(st.take_extra((size_t)n_q * k * 4, e));
-        blk_i = static_cast<int64_t *>(st.take_extra((size_t)n_q * k * 8, e));
-        return e == cudaSuccess ? FASTID_OK : scuda(ctx, e, "block lists");
-    };
-    // top-k of the block, folded into the running lists
+    auto setup = [](StreamState &) -> fastid_status { return FASTID_OK; };
+    // top-k of the first block, then every block's merged into it (which also
+    // starts each block's comparison at the running k-th scores)
     auto compare = [&](int64_t b, fastid_refdb &db, int64_t r0) -> fastid_status {
-        uint32_t *os = b == 0 ? out_scores_dev : blk_s;
-        int64_t *oi = b == 0 ? out_idx_dev : blk_i;
-        fastid_status st = fastid_topk(ctx, &db, queries_dev, ld_q, n_q, modes_dev, k, threshold, os, oi, stream);
-        if (st != FASTID_OK || b == 0) return st;
-        cudaError_t e = launch_topk_fold(out_scores_dev, out_idx_dev, blk_s, blk_i, r0, n_q, k, s);
-        if (e != cudaSuccess) return scuda(ctx, e, "fold");
-        ctx->launches += 1;
-        return FASTID_OK;
+        if (b == 0)
+            return fastid_topk(ctx, &db, queries_dev, ld_q, n_q, modes_dev, k, threshold, out_scores_dev, out_idx_dev,
+                               stream);
+        return fastid_topk_accumulate(ctx, &db, r0, queries_dev, ld_q, n_q, modes_dev, k, threshold, out_scores_dev,
+                                      out_idx_dev, stream);
     };
     return stream_blocks(ctx, R, n_q, k, s, setup, compare);
 }

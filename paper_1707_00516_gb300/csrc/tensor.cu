@@ -99,6 +99,7 @@ struct PanelDesc {
     int32_t n_kb;         // K stages of 128 operand bytes
     TcSched sc;
     const float *qconst;  // c_q per padded query row
+    int32_t *gcut;        // shared cut per padded query row, or nullptr (see TcLaunch)
     int32_t qspread;      // see spread_row_to_query
 };
 
@@ -539,6 +540,13 @@ __device__ __forceinline__ void store_scores(uint8_t *out, int64_t row_step, int
             }
         }
     }
+}
+
+// A shared cut (TcLaunch::gcut), which other CTAs lower meanwhile.
+__device__ __forceinline__ int32_t load_cut(const int32_t *p) {
+    int32_t v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
 }
 
 // Bounded wait that ignores the abort flag: used to drain this CTA's own
@@ -1100,14 +1108,29 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                             lr[i] = 0xFFFFFFFFu;
                         }
                     }
-                    float cut = ls[KM - 1] == NET_EMPTY ? cut0 : (float)ls[KM - 1] - cq;
+                    // the cut: below this list's k-th, and not above the shared one
+                    int32_t *gc = topk && P.gcut ? P.gcut + qr : nullptr;
+                    int32_t shared = gc ? load_cut(gc) : NET_EMPTY, newer = shared;
+                    float cut;
+                    auto set_cut = [&]() {
+                        cut = ls[KM - 1] == NET_EMPTY ? cut0 : (float)ls[KM - 1] - cq;
+                        if (shared != NET_EMPTY) cut = fminf(cut, (float)(shared + 1) - cq);
+                    };
+                    auto share_cut = [&]() {
+                        if (gc && ls[KM - 1] < shared) {
+                            shared = ls[KM - 1];
+                            atomicMin(gc, shared);
+                        }
+                    };
+                    set_cut();
                     uint32_t *queue = reinterpret_cast<uint32_t *>(sT) + row;  // entry i at i * TC_BM (see queue_insert)
                     int queued = 0;
                     int64_t qbase = rc * BN;
                     auto flush = [&]() {
                         queue_insert(queue, queued, qbase, ls, lr);
                         queued = 0;
-                        cut = ls[KM - 1] == NET_EMPTY ? cut0 : (float)ls[KM - 1] - cq;
+                        share_cut();
+                        set_cut();
                     };
                     for (int64_t rt = rc; rt < re; ++rt) {
                         const bool got = mbar_wait(smem_u32(&ctl->tfull[acc]), acc_phase, abort_flag, args.status, 6);
@@ -1118,6 +1141,13 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                         }
                         tc_fence_after();
                         const int64_t r0 = rt * BN;
+                        if (gc) {  // what the other slices had reached a tile ago
+                            if (newer < shared) {
+                                shared = newer;
+                                set_cut();
+                            }
+                            newer = load_cut(gc);
+                        }
                         if (topk && r0 + BN - qbase > TC_QSPAN) {  // the queues' reference window moves on
                             flush();
                             qbase = r0;
@@ -1184,8 +1214,9 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                                             xr = (uint32_t)(rch + j);
                                         }
                                         net_insert(ls, lr, xs, xr);
-                                        cut = ls[KM - 1] == NET_EMPTY ? cut0 : (float)ls[KM - 1] - cq;
+                                        set_cut();
                                     }
+                                    share_cut();
                                     continue;
                                 }
                             }
@@ -1385,16 +1416,28 @@ __device__ __forceinline__ void encode_query_row_f4(const uint64_t *__restrict__
     if (lane == 0) *qc = mis ? (float)pc : 0.f;
 }
 
+// Initial shared cut of operand row r, holding input query src (see SharedCut).
+// Scores are at most 65536, so a larger entry of a caller's list cuts nothing.
+__device__ __forceinline__ void init_cut(const SharedCut &cut, int64_t r, int64_t src, bool valid) {
+    int32_t c = NET_EMPTY;
+    if (valid && cut.run_s) {
+        const int64_t last = src * cut.k + cut.k - 1;
+        if (cut.run_i[last] >= 0 && cut.run_s[last] <= (uint32_t)FASTID_MAX_LOCI) c = (int32_t)cut.run_s[last];
+    }
+    cut.out[r] = c;
+}
+
 // Operand row r encodes input query spread_row_to_query(r, spread).
 __global__ void queries_e2m1_kernel(const uint64_t *__restrict__ q, int64_t ld_q, int64_t n_q, int32_t n_words,
                                     int32_t n_loci, const uint8_t *__restrict__ modes, int64_t n_q_pad,
                                     int32_t kbytes, uint8_t *__restrict__ out, float *__restrict__ qconst,
-                                    int64_t spread) {
+                                    int64_t spread, const SharedCut cut) {
     const int lane = threadIdx.x & 31;
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n_q_pad; r += warps_total) {
         const int64_t src = spread_row_to_query(r, spread);
         const bool valid = src < n_q;
+        if (cut.out && lane == 0) init_cut(cut, r, src, valid);
         encode_query_row_f4(valid ? q + src * ld_q : nullptr, valid && modes[src] == FASTID_MODE_MISMATCH, n_words,
                             n_loci, kbytes, out + r * (int64_t)kbytes, qconst + r, lane);
     }
@@ -1403,12 +1446,13 @@ __global__ void queries_e2m1_kernel(const uint64_t *__restrict__ q, int64_t ld_q
 __global__ void queries_e4m3_kernel(const uint64_t *__restrict__ q, int64_t ld_q, int64_t n_q, int32_t n_words,
                                     int32_t n_loci, const uint8_t *__restrict__ modes, int64_t n_q_pad,
                                     int32_t kpad, uint8_t *__restrict__ out, float *__restrict__ qconst,
-                                    uint32_t one, bool pk, int64_t spread) {
+                                    uint32_t one, bool pk, int64_t spread, const SharedCut cut) {
     const int lane = threadIdx.x & 31;
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n_q_pad; r += warps_total) {
         const int64_t src = spread_row_to_query(r, spread);
         const bool valid = src < n_q;
+        if (cut.out && lane == 0) init_cut(cut, r, src, valid);
         encode_query_row(valid ? q + src * ld_q : nullptr, valid && modes[src] == FASTID_MODE_MISMATCH, n_words,
                          n_loci, kpad, out + r * (int64_t)kpad, qconst + r, lane, one, pk);
     }
@@ -1421,6 +1465,7 @@ __global__ void prep_jobs_kernel(const PrepJob *__restrict__ jobs, int64_t n_job
     for (int64_t j = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < n_jobs; j += warps_total) {
         const PrepJob jb = jobs[j];
         const bool mis = jb.src != nullptr && *jb.mode == FASTID_MODE_MISMATCH;
+        if (lane == 0) *jb.gc = NET_EMPTY;
         if (jb.f4)
             encode_query_row_f4(jb.src, mis, jb.n_words, jb.n_loci, jb.kpad, jb.dst, jb.qc, lane);
         else
@@ -1487,11 +1532,11 @@ cudaError_t launch_refs_e2m1(const uint64_t *packed, int64_t ld64, int64_t n_src
 
 cudaError_t launch_queries_e2m1(const uint64_t *q, int64_t ld_q, int64_t n_q, int32_t n_words, int32_t n_loci,
                                 const uint8_t *modes, int64_t n_q_pad, int32_t kbytes, uint8_t *out, float *qconst,
-                                int64_t spread, cudaStream_t s) {
+                                int64_t spread, const SharedCut &cut, cudaStream_t s) {
     int64_t blocks = (n_q_pad + 7) / 8;
     if (blocks > 65535) blocks = 65535;
     queries_e2m1_kernel<<<(unsigned)blocks, 256, 0, s>>>(q, ld_q, n_q, n_words, n_loci, modes, n_q_pad, kbytes, out,
-                                                         qconst, spread);
+                                                         qconst, spread, cut);
     return cudaGetLastError();
 }
 
@@ -1507,11 +1552,11 @@ cudaError_t launch_refs_e4m3(const uint64_t *packed, int64_t ld64, int64_t n_src
 
 cudaError_t launch_queries_e4m3(const uint64_t *q, int64_t ld_q, int64_t n_q, int32_t n_words, int32_t n_loci,
                                 const uint8_t *modes, int64_t n_q_pad, int32_t kpad, uint8_t *out, float *qconst,
-                                bool half, int64_t spread, cudaStream_t s) {
+                                bool half, int64_t spread, const SharedCut &cut, cudaStream_t s) {
     int64_t blocks = (n_q_pad + 7) / 8;
     if (blocks > 65535) blocks = 65535;
     queries_e4m3_kernel<<<(unsigned)blocks, 256, 0, s>>>(q, ld_q, n_q, n_words, n_loci, modes, n_q_pad, kpad, out,
-                                                         qconst, half ? 0x30u : 0x38u, half, spread);
+                                                         qconst, half ? 0x30u : 0x38u, half, spread, cut);
     return cudaGetLastError();
 }
 
@@ -1622,6 +1667,7 @@ cudaError_t launch_tensor_multi(int bn, const TcLaunch &L, cudaStream_t s) {
         a.panel[p].n_kb = L.kpad[p] / TC_BK;
         a.panel[p].sc = L.sched[p];
         a.panel[p].qconst = L.qconst[p];
+        a.panel[p].gcut = L.gcut[p];
         a.panel[p].qspread = L.qspread[p];
         a.order[p] = L.order[p];
     }
