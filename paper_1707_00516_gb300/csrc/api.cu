@@ -1,5 +1,6 @@
 // C ABI of the library (declared in include/fastid.h): argument checks,
 // context and database ownership, scratch memory, and launch sequencing.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -12,6 +13,7 @@
 
 using namespace fastid;
 
+#include "few.h"
 #include "internal.h"
 
 namespace {
@@ -583,9 +585,72 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
     return FASTID_OK;
 }
 
+bool use_few(int op, int64_t n_q, int32_t n_loci, int32_t k, FewShape *S) {
+    return op == OP_FP4_PACKED && few_shape(n_q, n_loci, k, S);
+}
+
+// Few-query launch of a top-k call (few.cu) over packed rows.
+fastid_status topk_few(fastid_ctx *ctx, const fastid_refdb *db, const FewShape &S, const uint64_t *q, int64_t ld_q,
+                       int64_t n_q, const uint8_t *modes, int32_t k, uint32_t threshold, uint32_t *out_scores,
+                       int64_t *out_idx, bool accumulate, int64_t ref_offset, cudaStream_t s);
+
 uint32_t clamp_threshold(uint32_t t, int32_t n_loci) {
     if (t == 0xFFFFFFFFu) return t;
     return t > (uint32_t)n_loci ? (uint32_t)n_loci : t;
+}
+
+fastid_status topk_few(fastid_ctx *ctx, const fastid_refdb *db, const FewShape &S, const uint64_t *q, int64_t ld_q,
+                       int64_t n_q, const uint8_t *modes, int32_t k, uint32_t threshold, uint32_t *out_scores,
+                       int64_t *out_idx, bool accumulate, int64_t ref_offset, cudaStream_t s) {
+    Scratch scr(ctx, s);
+    const int64_t rows = S.ncols;
+    const int32_t slices = (int32_t)std::min<int64_t>((db->n_refs + 127) / 128, ctx->grid_tensor);
+    Carver cv;
+    const size_t o_a = cv.take<uint8_t>((size_t)rows * S.n_kb * 128);
+    const size_t o_c = cv.take<float>((size_t)rows);
+    const size_t o_g = cv.take<int32_t>((size_t)rows);
+    const size_t o_u = cv.take<int32_t>((size_t)rows * slices);
+    const size_t o_p = cv.take<uint64_t>((size_t)slices * TC_TILE_Q * k);
+    FASTID_CUDA(ctx, scr.alloc(cv.off));
+    FewLaunch F;
+    memset(&F, 0, sizeof F);
+    F.q = q;
+    F.ld_q = ld_q;
+    F.n_q = n_q;
+    F.n_words = db->n_words64;
+    F.n_loci = db->n_loci;
+    F.modes = modes;
+    F.operand = at<uint8_t>(scr.p, o_a);
+    F.qconst = at<float>(scr.p, o_c);
+    F.cut = SharedCut{at<int32_t>(scr.p, o_g), accumulate ? out_scores : nullptr, accumulate ? out_idx : nullptr, k};
+    F.packed = db->packed;
+    F.n_pad = db->n_pad;
+    F.ld64 = db->ld64;
+    F.n_refs = db->n_refs;
+    F.k = k;
+    F.threshold = clamp_threshold(threshold, db->n_loci);
+    F.slices = slices;
+    F.pub = at<int32_t>(scr.p, o_u);
+    F.partial = at<uint64_t>(scr.p, o_p);
+    F.status = ctx->dev_status;
+    FASTID_CUDA(ctx, launch_few_seed(F, S, s));
+    MainTimer tm(ctx, s);
+    FASTID_CUDA(ctx, launch_few(F, S, s));
+    tm.done();
+    TcLaunch L;  // what the merge needs: slice y's lists in slot y
+    memset(&L, 0, sizeof L);
+    L.n_panels = 1;
+    L.k = k;
+    L.n_slots = slices;
+    L.status = ctx->dev_status;
+    L.sched[0].n_qq = 1;
+    L.sched[0].a = 1;
+    L.sched[0].b = slices;
+    L.sched[0].tpx = 1;
+    L.sched[0].t_tpx = 1;
+    FASTID_CUDA(ctx, launch_merge_sched(F.partial, L, nullptr, n_q, out_scores, out_idx, s, accumulate, ref_offset));
+    count_launches(ctx, 3);
+    return FASTID_OK;
 }
 
 }  // namespace
@@ -650,6 +715,10 @@ fastid_status fastid_topk(fastid_ctx *ctx, const fastid_refdb *db, const uint64_
     if (n_q == 0) return FASTID_OK;
     FASTID_CUDA(ctx, cudaSetDevice(ctx->device));
     cudaStream_t s = (cudaStream_t)stream;
+    FewShape few;
+    if (use_few(tensor, n_q, db->n_loci, k, &few))
+        return topk_few(ctx, db, few, queries_dev, ld_q, n_q, modes_dev, k, threshold, out_scores_dev, out_idx_dev,
+                        false, 0, s);
     Scratch scr(ctx, s);
     if (tensor) {
         TensorPrep tp;
@@ -701,6 +770,10 @@ fastid_status fastid_topk_accumulate(fastid_ctx *ctx, const fastid_refdb *db, in
     if (n_q == 0) return FASTID_OK;
     FASTID_CUDA(ctx, cudaSetDevice(ctx->device));
     cudaStream_t s = (cudaStream_t)stream;
+    FewShape few;
+    if (use_few(op, n_q, db->n_loci, k, &few))
+        return topk_few(ctx, db, few, queries_dev, ld_q, n_q, modes_dev, k, threshold, run_scores_dev, run_idx_dev,
+                        true, ref_offset, s);
     Scratch scr(ctx, s);
     if (op) {
         TensorPrep tp;

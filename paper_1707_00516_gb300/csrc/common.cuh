@@ -261,9 +261,10 @@ cudaError_t launch_queries_e4m3(const uint64_t *q, int64_t ld_q, int64_t n_q, in
                                 const uint8_t *modes, int64_t n_q_pad, int32_t kpad, uint8_t *out, float *qconst,
                                 bool half, int64_t spread, const SharedCut &cut, cudaStream_t s);
 // TMA map over packed rows for packed-reference (PK) launches: boxes of 2
-// words x 256 rows (FP8 stages) or 4 words x 224 rows (FP4 stages).
+// words x 256 rows (FP8 stages) or 4 words x 224 rows (FP4 stages); 8 words x
+// 128 rows with a 64-byte swizzle for few-query launches.
 cudaError_t make_packed_map(CUtensorMap *map, const uint64_t *packed, int64_t rows, int64_t ld64, int box_words = 2,
-                            int box_rows = 256);
+                            int box_rows = 256, bool swizzle64 = false);
 // FP4 form: reference tile (224), operand row bytes of n_loci (loci padded to
 // 256, two per byte), the database's FP4 copy and the query operand.
 int tensor_tile_r4();

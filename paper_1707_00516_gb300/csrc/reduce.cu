@@ -3,32 +3,11 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "keys.cuh"
 
 namespace fastid {
 
 namespace {
-
-__device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
-    uint32_t lo = __shfl_sync(0xffffffffu, (uint32_t)v, src);
-    uint32_t hi = __shfl_sync(0xffffffffu, (uint32_t)(v >> 32), src);
-    return ((uint64_t)hi << 32) | lo;
-}
-__device__ __forceinline__ uint64_t shfl_xor64(uint64_t v, int m) {
-    uint32_t lo = __shfl_xor_sync(0xffffffffu, (uint32_t)v, m);
-    uint32_t hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(v >> 32), m);
-    return ((uint64_t)hi << 32) | lo;
-}
-__device__ __forceinline__ uint64_t warp_merge32(uint64_t a, uint64_t b, int lane) {
-    uint64_t br = shfl64(b, 31 - lane);
-    uint64_t v = a < br ? a : br;
-#pragma unroll
-    for (int j = 16; j > 0; j >>= 1) {
-        uint64_t p = shfl_xor64(v, j);
-        bool lower = (lane & j) == 0;
-        v = lower ? (v < p ? v : p) : (v < p ? p : v);
-    }
-    return v;
-}
 
 // Merge of one query's lists by W warps (a power of two, all in one block).
 // A list is k ascending keys, one per lane; list i is load(i), KEY_EMPTY on

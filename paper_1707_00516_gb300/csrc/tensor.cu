@@ -36,7 +36,7 @@
 
 #include <cstring>
 
-#include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace fastid {
 
@@ -57,14 +57,12 @@ __host__ __device__ constexpr uint32_t pk_stage_bytes(int bn, bool f4) { return 
 // TC_SF_COL.. (A's from TC_SF_COL, B's from TC_SF_COL + 16), all lanes.
 constexpr int TC_BN4 = 224;
 constexpr uint32_t TC_SF_COL = 448;
-constexpr uint32_t TC_SF_UNIT = 0x7F7F7F7Fu;  // four ue8m0 bytes of 2^0
 // Full-matrix launches: each epilogue warp turns a 32 x 32 block of scores
 // from thread-per-query to query-major through a buffer of 32 rows of 36
 // words (16-byte rows; a quarter-warp's 16-byte accesses meet every bank once
 // both ways).
 constexpr int SC_LD = 36;
 constexpr uint32_t SC_BYTES = 4 * 32 * SC_LD * 4;
-constexpr uint64_t WAIT_NS = 2000000000ull;     // 2 s per wait
 constexpr uint64_t RENDEZVOUS_NS = 50000000ull;  // 50 ms per panel entry, then go on alone
 
 // Kernel variants: references per tile (the MMA's N) and pipeline depth (as
@@ -130,179 +128,6 @@ struct TensorArgs {
     unsigned int *arrive;  // panel-entry counters (see the producer), or nullptr
 };
 
-// ---- PTX wrappers --------------------------------------------------------
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint64_t globaltimer() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait; returns false (and records a timeout) if the phase does not
-// complete within WAIT_NS or if another thread of the CTA already gave up.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
-                                          uint32_t *status, uint32_t site) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = globaltimer();
-    for (uint32_t it = 1;; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((it & 255) == 0) {
-            if (*abort_flag) return false;
-            if (globaltimer() - t0 > WAIT_NS) {
-                *abort_flag = 1;
-                atomicOr(status, ST_TIMEOUT);
-                atomicExch(status + 1, site);
-                return false;
-            }
-        }
-    }
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int32_t x,
-                                            int32_t y) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-
-// Multicast variant: the box lands at the same shared-memory offset in every
-// CTA of ctamask and completes bytes on the mbarrier at the same offset there.
-__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const CUtensorMap *map, uint32_t bar, int32_t x,
-                                               int32_t y, uint16_t ctamask) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster "
-        "[%0], [%1, {%2, %3}], [%4], %5;"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(ctamask)
-        : "memory");
-}
-
-// L2 prefetch of one box (no shared-memory destination, no completion).
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *map, int32_t x, int32_t y) {
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
-                 ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y)
-                 : "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// Every thread of every CTA in the cluster.
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// The MMA issuer is a whole converged warp: every lane runs its loop and its
-// waits, and one lane, picked by elect.sync (the same lane every time in a
-// converged warp), issues each tcgen05.mma and tcgen05.commit -- a commit
-// tracks the operations of the thread that executes it.  A single lane
-// running the loop alone, inside a branch the rest of its warp skips, left
-// the tensor pipe idle for ~180 of every ~630 cycles of an FP4 stage.
-#define FASTID_ELECT "elect.sync _|e, 0xffffffff;\n\t"
-
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("{\n\t.reg .pred e;\n\t" FASTID_ELECT
-                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
-                 : "memory");
-}
-
-// Arrive (when the elected lane's prior tcgen05 operations complete) on the
-// mbarrier at the same offset in every CTA of ctamask.
-__device__ __forceinline__ void tc_commit_mc(uint32_t bar, uint16_t ctamask) {
-    asm volatile(
-        "{\n\t.reg .pred e;\n\t" FASTID_ELECT
-        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
-            bar),
-        "h"(ctamask)
-        : "memory");
-}
-
-// ---- 2-SM (cta_group::2) forms: the MMA of a CTA pair issued by its even
-// CTA, M = 256 rows (128 in each CTA's shared memory and TMEM), the
-// reference operand split along N (half in each CTA's shared memory) ----
-
-// Address of the same shared-memory object in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t mapa_rank(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-
-// Arrive on an mbarrier of (possibly) another CTA of the cluster, release
-// ordering at cluster scope (bar: a shared::cluster address).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// TMA load into this CTA's shared memory whose completion counts on the
-// mbarrier `bar` of either CTA of the pair (a shared::cluster address).
-__device__ __forceinline__ void tma_load_2d_cg2(uint32_t dst, const CUtensorMap *map, uint32_t bar, int32_t x,
-                                                int32_t y) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 "
-        "[%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-
-// Arrive on the mbarrier at the same offset in every CTA of ctamask when the
-// elected lane's prior cta_group::2 tcgen05 operations complete.
-__device__ __forceinline__ void tc_commit_cg2_mc(uint32_t bar, uint16_t ctamask) {
-    asm volatile(
-        "{\n\t.reg .pred e;\n\t" FASTID_ELECT
-        "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
-            bar),
-        "h"(ctamask)
-        : "memory");
-}
-
-__device__ __forceinline__ void tc_commit_cg2(uint32_t bar) {
-    asm volatile("{\n\t.reg .pred e;\n\t" FASTID_ELECT
-                 "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
-                 : "memory");
-}
-
-// 32 lanes x 16 consecutive 32-bit columns, every column the value v.
-__device__ __forceinline__ void tmem_fill16(uint32_t taddr, uint32_t v) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
-        "r"(v)
-        : "memory");
-}
-
 // The 4 MMAs of one 128-byte K stage into accumulator d: operand descriptors
 // +0, +2, +4, +6 (32 bytes of K each in the address field), the first MMA
 // accumulating only when acc != 0, the others always; one asm block with its
@@ -353,58 +178,6 @@ __device__ __forceinline__ void mma_stage4(uint32_t d, uint64_t ad, uint64_t bd,
     }
 }
 
-// 32 lanes x one 32-bit column (every lane its own row).
-__device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
-    uint32_t v;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    return v;
-}
-
-// 32 lanes x 32 consecutive 32-bit columns.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
-          "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
-          "=r"(v[30]), "=r"(v[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, rows of 128
-// bytes, 8-row groups 1024 bytes apart (tile base 1024-byte aligned).
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);  // start address
-    d |= (uint64_t)1 << 16;                    // leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)(1024 >> 4) << 32;          // stride byte offset: 8 rows x 128 B
-    d |= (uint64_t)1 << 46;                    // descriptor version
-    d |= (uint64_t)2 << 61;                    // 128-byte swizzle
-    return d;
-}
-
-// Instruction descriptor, kind::f8f6f4: D = F32, A = B = E4M3, both K-major,
-// N = 256, M = 128.
-__host__ __device__ constexpr uint32_t idesc_f8(int m, int n) {
-    return (1u << 4)                      // D format: F32
-           | (0u << 7) | (0u << 10)       // A, B format: E4M3
-           | ((uint32_t)(n >> 3) << 17)   // N >> 3
-           | ((uint32_t)(m >> 4) << 24);  // M >> 4
-}
-
-// Instruction descriptor, kind::mxf4 (block-scaled): B scale-factor id 0
-// (bits 4-5), A = B = E2M1 (1 at bits 7 and 10), both K-major, N >> 3 at bit
-// 17, scale type UE8M0 (bit 23), M >> 4 at bit 24 (for M = 128 the same bit
-// as M >> 7 at bit 27), A scale-factor id 0 (bits 29-30), K = 64 (bit 31 = 0).
-__host__ __device__ constexpr uint32_t idesc_mxf4(int m, int n) {
-    return (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (1u << 23) | ((uint32_t)(m >> 4) << 24);
-}
-
 // Per-thread top-k list held in registers, ascending by score; entries of
 // equal score keep arrival order (references arrive in increasing order, so
 // the earlier entry has the lower index).  Inserting (xs, xr) is a fixed
@@ -415,7 +188,6 @@ __host__ __device__ constexpr uint32_t idesc_mxf4(int m, int n) {
 // nothing displaces, so the k kept entries sit in slots KM-k .. KM-1 and the
 // k-th smallest is always slot KM-1 (static register indices only).
 constexpr int TC_KMAX = 32;
-constexpr int32_t NET_EMPTY = 0x7fffffff;
 constexpr int32_t NET_HOLD = (int32_t)0x80000000;
 
 template <int KM>
@@ -444,9 +216,6 @@ __device__ __forceinline__ void net_insert(int32_t (&ls)[KM], uint32_t (&lr)[KM]
 // the lower reference first; one that no longer beats the list changes
 // nothing.  The cut is that of the last insertion, so a deeper queue lets more
 // late candidates in: with k = 16 and 8 entries about a fifth more.
-constexpr int TC_QBITS = 15;  // 17 bits hold any score (N <= 65536)
-constexpr int64_t TC_QSPAN = 1ll << TC_QBITS;
-
 template <int KM>
 __device__ __forceinline__ void queue_insert(const uint32_t *queue, int queued, int64_t qbase, int32_t (&ls)[KM],
                                              uint32_t (&lr)[KM]) {
@@ -538,26 +307,6 @@ __device__ __forceinline__ void store_scores(uint8_t *out, int64_t row_step, int
                 else
                     *reinterpret_cast<uint32_t *>(p) = b[i * SC_LD];
             }
-        }
-    }
-}
-
-// A shared cut (TcLaunch::gcut), which other CTAs lower meanwhile.
-__device__ __forceinline__ int32_t load_cut(const int32_t *p) {
-    int32_t v;
-    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-
-// Bounded wait that ignores the abort flag: used to drain this CTA's own
-// asynchronous copies and MMAs before it exits.
-__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity, uint32_t *status, uint32_t site) {
-    const uint64_t t0 = globaltimer();
-    while (!mbar_try_wait(bar, parity)) {
-        if (globaltimer() - t0 > WAIT_NS) {
-            atomicOr(status, ST_TIMEOUT);
-            atomicExch(status + 1, site);
-            return;
         }
     }
 }
@@ -1564,7 +1313,7 @@ cudaError_t launch_queries_e4m3(const uint64_t *q, int64_t ld_q, int64_t n_q, in
 // boxes of box_words words (2 = 128 loci for FP8 stages, 4 = 256 for FP4) x
 // box_rows references, unswizzled.
 cudaError_t make_packed_map(CUtensorMap *map, const uint64_t *packed, int64_t rows, int64_t ld64, int box_words,
-                            int box_rows) {
+                            int box_rows, bool swizzle64) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return cudaErrorNotSupported;
     cuuint64_t dims[2] = {(cuuint64_t)ld64, (cuuint64_t)rows};
@@ -1572,7 +1321,8 @@ cudaError_t make_packed_map(CUtensorMap *map, const uint64_t *packed, int64_t ro
     cuuint32_t box[2] = {(cuuint32_t)box_words, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<uint64_t *>(packed), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
