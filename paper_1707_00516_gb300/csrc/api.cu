@@ -152,9 +152,11 @@ fastid_status fastid_create(fastid_ctx **out, int32_t device) {
         delete ctx;
         return e == cudaErrorMemoryAllocation ? FASTID_ENOMEM : FASTID_ECUDA;
     }
-    ctx->grid_topk = plain_grid_target(EPI_TOPK, device);
-    ctx->grid_hits = plain_grid_target(EPI_HITS, device);
-    ctx->grid_scores = plain_grid_target(EPI_SCORES32, device);
+    for (int t = 0; t < PL_TILES; ++t) {
+        ctx->grid_plain[0][t] = plain_grid_target(EPI_TOPK, 128 >> t, device);
+        ctx->grid_plain[1][t] = plain_grid_target(EPI_HITS, 128 >> t, device);
+        ctx->grid_plain[2][t] = plain_grid_target(EPI_SCORES32, 128 >> t, device);
+    }
     ctx->grid_tensor = tensor_grid_target(device);
     ctx->pair_clusters = tensor_pair_clusters(device);
     *out = ctx;
@@ -476,9 +478,9 @@ namespace {
 // and coefficients (+ `extra` bytes), query preparation.
 fastid_status prepare(fastid_ctx *ctx, const fastid_refdb *db, const uint64_t *q, int64_t ld_q, int64_t n_q,
                       const uint8_t *modes, cudaStream_t s, Scratch &scr, size_t extra, size_t *extra_off,
-                      PreparedQueries *pq) {
+                      PreparedQueries *pq, const Partition &part) {
     const int64_t ld32 = db->ld64 * 2;
-    pq->n_q_pad = round_up(n_q, PL_TQ);
+    pq->n_q_pad = (int64_t)part.n_qt * part.tile_q;
     Carver cv;
     size_t o_q = cv.take<uint32_t>((size_t)pq->n_q_pad * ld32);
     size_t o_c = cv.take<QueryCoef>((size_t)pq->n_q_pad);
@@ -691,8 +693,8 @@ fastid_status fastid_scores(fastid_ctx *ctx, const fastid_refdb *db, const uint6
         return FASTID_OK;
     }
     PreparedQueries pq;
-    if ((st = prepare(ctx, db, queries_dev, ld_q, n_q, modes_dev, s, scr, 0, &xo, &pq))) return st;
-    Partition part = make_partition((int32_t)(pq.n_q_pad / PL_TQ), db->n_pad / PL_TR, ctx->grid_scores);
+    const Partition part = fastid::plain_partition(ctx, EPI_SCORES32, n_q, db->n_pad);
+    if ((st = prepare(ctx, db, queries_dev, ld_q, n_q, modes_dev, s, scr, 0, &xo, &pq, part))) return st;
     MainTimer tm(ctx, s);
     FASTID_CUDA(ctx, launch_plain(out_bytes == 2 ? EPI_SCORES16 : EPI_SCORES32, (const uint32_t *)db->packed,
                                   db->norms, db->n_refs, db->ld64 * 2, db->n_words64 * 2, pq.q32, pq.coef, n_q,
@@ -738,12 +740,12 @@ fastid_status fastid_topk(fastid_ctx *ctx, const fastid_refdb *db, const uint64_
         count_launches(ctx, 2);
         return FASTID_OK;
     }
-    const int64_t n_q_pad = round_up(n_q, PL_TQ);
-    Partition part = make_partition((int32_t)(n_q_pad / PL_TQ), db->n_pad / PL_TR, ctx->grid_topk);
-    const size_t partial_elems = (size_t)part.grid * part.max_seg * PL_TQ * k;
+    const Partition part = fastid::plain_partition(ctx, EPI_TOPK, n_q, db->n_pad);
+    const size_t partial_elems = (size_t)part.grid * part.max_seg * part.tile_q * k;
     PreparedQueries pq;
     size_t xo;
-    if ((st = prepare(ctx, db, queries_dev, ld_q, n_q, modes_dev, s, scr, partial_elems * 8, &xo, &pq))) return st;
+    if ((st = prepare(ctx, db, queries_dev, ld_q, n_q, modes_dev, s, scr, partial_elems * 8, &xo, &pq, part)))
+        return st;
     uint64_t *partial = at<uint64_t>(scr.p, xo);
     MainTimer tm(ctx, s);
     FASTID_CUDA(ctx, launch_plain(EPI_TOPK, (const uint32_t *)db->packed, db->norms, db->n_refs, db->ld64 * 2,
@@ -795,13 +797,12 @@ fastid_status fastid_topk_accumulate(fastid_ctx *ctx, const fastid_refdb *db, in
         return FASTID_OK;
     }
     // plain form: the call's lists in scratch, then folded
-    const int64_t n_q_pad = round_up(n_q, PL_TQ);
-    Partition part = make_partition((int32_t)(n_q_pad / PL_TQ), db->n_pad / PL_TR, ctx->grid_topk);
-    const size_t partial_elems = (size_t)part.grid * part.max_seg * PL_TQ * k;
+    const Partition part = fastid::plain_partition(ctx, EPI_TOPK, n_q, db->n_pad);
+    const size_t partial_elems = (size_t)part.grid * part.max_seg * part.tile_q * k;
     PreparedQueries pq;
     size_t xo;
     if ((st = prepare(ctx, db, queries_dev, ld_q, n_q, modes_dev, s, scr, partial_elems * 8 + (size_t)n_q * k * 12 + 512,
-                      &xo, &pq)))
+                      &xo, &pq, part)))
         return st;
     uint64_t *partial = at<uint64_t>(scr.p, xo);
     uint8_t *lists = reinterpret_cast<uint8_t *>(partial + partial_elems);
@@ -862,6 +863,14 @@ fastid_status check_topk_args(fastid_ctx *ctx, const fastid_refdb *db, const uin
     if (k < 1 || k > FASTID_MAX_K) return fail(ctx, FASTID_EINVAL, "k out of range: %d", k);
     if (n_q > 0 && (!out_scores || !out_idx)) return fail(ctx, FASTID_EINVAL, "output is NULL");
     return FASTID_OK;
+}
+
+Partition plain_partition(const fastid_ctx *ctx, int epi, int64_t n_q, int64_t n_pad) {
+    const int tile = plain_tile_q(n_q);
+    int t = 0;
+    while ((128 >> t) != tile) ++t;
+    const int kind = epi == EPI_TOPK ? 0 : epi == EPI_HITS ? 1 : 2;
+    return make_partition(tile, n_q, n_pad / PL_TR, ctx->grid_plain[kind][t]);
 }
 
 MainTimer::MainTimer(fastid_ctx *c, cudaStream_t st) : ctx(c), s(st) {
@@ -933,8 +942,8 @@ fastid_status compare_append(fastid_ctx *ctx, const fastid_refdb *db, const uint
     }
     PreparedQueries pq;
     size_t xo;
-    if ((st = prepare(ctx, db, queries_dev, ld_q, n_q, modes_dev, s, scr, 0, &xo, &pq))) return st;
-    Partition part = make_partition((int32_t)(pq.n_q_pad / PL_TQ), db->n_pad / PL_TR, ctx->grid_hits);
+    const Partition part = plain_partition(ctx, EPI_HITS, n_q, db->n_pad);
+    if ((st = prepare(ctx, db, queries_dev, ld_q, n_q, modes_dev, s, scr, 0, &xo, &pq, part))) return st;
     MainTimer tm(ctx, s);
     FASTID_CUDA(ctx, launch_plain(EPI_HITS, (const uint32_t *)db->packed, db->norms, db->n_refs, db->ld64 * 2,
                                   db->n_words64 * 2, pq.q32, pq.coef, n_q, threshold, 1, nullptr, 0, capacity,

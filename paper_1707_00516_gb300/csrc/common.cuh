@@ -16,10 +16,10 @@ enum : uint32_t {
     ST_DEVICE = 4u,    // a device-side consistency check failed
 };
 
-// Plain-form tile: 128 references x 128 queries per CTA, K staged in chunks of
-// KC 32-bit words.
+// Plain-form tile: 128 references x up to 128 queries (Partition::tile_q) per
+// CTA, K staged in chunks of KC 32-bit words.
 constexpr int PL_TR = 128;       // references per tile
-constexpr int PL_TQ = 128;       // queries per tile
+constexpr int PL_TILES = 4;      // query tile heights: 128, 64, 32, 16
 constexpr int PL_KC = 16;        // u32 words per K stage
 constexpr int PL_THREADS = 256;  // 16 x 16 threads, 8 x 8 outputs each
 constexpr int ROW_ALIGN = 256;   // database rows are padded to this multiple (both forms' tiles)
@@ -43,14 +43,17 @@ struct Partition {
     int64_t n_rt;      // reference tiles
     int32_t grid;      // G
     int32_t max_seg;   // max query-tile segments per CTA
+    int32_t tile_q;    // queries a tile
 };
 
 __host__ __device__ inline int64_t part_begin(const Partition &p, int64_t c) {
     return (c * p.n_units) / p.grid;
 }
 
-__host__ inline Partition make_partition(int32_t n_qt, int64_t n_rt, int32_t grid_target) {
+__host__ inline Partition make_partition(int32_t tile_q, int64_t n_q, int64_t n_rt, int32_t grid_target) {
     Partition p;
+    const int32_t n_qt = (int32_t)((n_q + tile_q - 1) / tile_q);
+    p.tile_q = tile_q;
     p.n_qt = n_qt;
     p.n_rt = n_rt;
     p.n_units = (int64_t)n_qt * n_rt;
@@ -225,7 +228,8 @@ cudaError_t launch_plain(int epi, const uint32_t *refs32, const uint32_t *ref_no
                          int64_t *hit_r, uint32_t *hit_score, unsigned long long *hit_count,
                          uint64_t *partial, const Partition &part, uint32_t *status,
                          cudaStream_t s);
-int plain_grid_target(int epi, int device);
+int plain_tile_q(int64_t n_q);  // query tile height for a call
+int plain_grid_target(int epi, int tile_q, int device);
 cudaError_t launch_topk_merge(const uint64_t *partial, const Partition &part, int64_t n_q,
                               int32_t k, uint32_t *out_scores, int64_t *out_idx, cudaStream_t s);
 // Hit-list finish (reduce.cu).  The scratch of a hit call holds the device

@@ -30,7 +30,8 @@ struct fastid_ctx {
     int sms = 0;
     cudaMemPool_t pool = nullptr;
     uint32_t *dev_status = nullptr;  // [8]: the live word [0..3], a snapshot [4..7] (fastid_sync_status)
-    int grid_topk = 0, grid_hits = 0, grid_scores = 0, grid_tensor = 0;
+    int grid_plain[3][fastid::PL_TILES] = {};  // plain CTAs resident at once: top-k, hits, scores; by tile height
+    int grid_tensor = 0;
     int pair_clusters = 0;  // resident 2-CTA clusters of the paired tensor kernel (0: never pair)
     std::string last_error;
     // profiling (fastid_profile)
@@ -90,6 +91,10 @@ __host__ __device__ inline bool op_f4(int op) { return op == OP_FP4 || op == OP_
 // copy wins from two query tiles on.
 constexpr int64_t AUTO_FP4_PACKED_MAX_Q = 128;
 int pick_operand(int form, bool has_fp8, bool has_fp4, int64_t n_q, bool slots16 = true);
+
+// Work partition of a plain-form launch over n_pad padded references; its
+// query operand has n_qt * tile_q rows.
+Partition plain_partition(const fastid_ctx *ctx, int epi, int64_t n_q, int64_t n_pad);
 
 // Argument checks of the top-k entry points (fastid_topk, fastid_topk_noalloc,
 // fastid_topk_accumulate): the shared query arguments, k, and the two output

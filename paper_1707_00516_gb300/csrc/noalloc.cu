@@ -79,12 +79,12 @@ extern "C" fastid_status fastid_topk_noalloc(fastid_ctx *ctx, const fastid_refdb
 
     // Scratch layout: padded queries, coefficients, per-segment top-k lists.
     const int64_t ld32 = db->ld64 * 2;
-    const int64_t n_q_pad = round_up(n_q, PL_TQ);
-    Partition part = make_partition((int32_t)(n_q_pad / PL_TQ), db->n_pad / PL_TR, ctx->grid_topk);
+    const Partition part = plain_partition(ctx, EPI_TOPK, n_q, db->n_pad);
+    const int64_t n_q_pad = (int64_t)part.n_qt * part.tile_q;
     const int64_t off_q = 0;
     const int64_t off_c = round_up(off_q + n_q_pad * ld32 * (int64_t)sizeof(uint32_t), 256);
     const int64_t off_p = round_up(off_c + n_q_pad * (int64_t)sizeof(QueryCoef), 256);
-    const int64_t need = off_p + (int64_t)part.grid * part.max_seg * PL_TQ * k * (int64_t)sizeof(uint64_t);
+    const int64_t need = off_p + (int64_t)part.grid * part.max_seg * part.tile_q * k * (int64_t)sizeof(uint64_t);
     if (need > (int64_t)FASTID_NOALLOC_SCRATCH_BYTES) {
         char buf[256];
         snprintf(buf, sizeof buf,

@@ -13,9 +13,11 @@
 //     mode 0: a = 2, b = |Q|  ->  |R| + |Q| - 2G = popc(R XOR Q)
 //     mode 1: a = 1, b = 0    ->  |R| - G       = popc(R AND NOT Q)  (Eq. 1)
 //
-// CTA tile: 128 references x 128 queries, 256 threads, each thread owns 8
-// references (rows tr + 16 i) and 8 queries (rows tq + 16 j) of the tile;
-// two CTAs an SM.
+// CTA tile: 128 references x TQ queries, 256 threads, each thread owns 8
+// references (rows tr + 16 i) and JQ = TQ / 16 queries (rows tq + 16 j) of the
+// tile; two CTAs an SM at TQ = 128, more below.  TQ is 128, 64, 32 or 16, the
+// one that pads the call's queries least (plain_tile_q): a tile costs its full
+// height whatever part of it is queries.
 // The grid is persistent: CTA c walks the units [c U / G, (c+1) U / G) of the
 // query-tile-major list of (query tile, reference tile) units, so within one
 // query tile a CTA sees references in increasing order.
@@ -61,11 +63,12 @@ struct PlainArgs {
     uint32_t two;  // 2 (see and_popc8)
 };
 
+template <int TQ>
 struct TopkSmem {
-    uint64_t list[PL_TQ][FASTID_MAX_K];  // sorted ascending; KEY_EMPTY pads
-    uint64_t stage[PL_TQ][STG];
-    uint64_t cut[PL_TQ];
-    int32_t cnt[PL_TQ];
+    uint64_t list[TQ][FASTID_MAX_K];  // sorted ascending; KEY_EMPTY pads
+    uint64_t stage[TQ][STG];
+    uint64_t cut[TQ];
+    int32_t cnt[TQ];
     int32_t ovf[2];
 };
 
@@ -123,13 +126,15 @@ __device__ __forceinline__ uint4 lds128_once(const uint32_t *p) {
     return v;
 }
 
-template <int EPI>
-__global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs args) {
+template <int EPI, int JQ>
+__global__ void __launch_bounds__(PL_THREADS, JQ > 2 ? 2 : 3) plain_kernel(const PlainArgs args) {
+    constexpr int TQ = 16 * JQ;
+    constexpr int JC = JQ < 4 ? JQ : 4;  // query columns a step
     extern __shared__ __align__(16) uint8_t smem_raw[];
     uint32_t(*sR)[PL_TR][KCP] = reinterpret_cast<uint32_t(*)[PL_TR][KCP]>(smem_raw);
-    uint32_t(*sQ)[PL_TQ][KCP] =
-        reinterpret_cast<uint32_t(*)[PL_TQ][KCP]>(smem_raw + 2 * PL_TR * KCP * sizeof(uint32_t));
-    TopkSmem *tk = reinterpret_cast<TopkSmem *>(smem_raw + 2 * (PL_TR + PL_TQ) * KCP * sizeof(uint32_t));
+    uint32_t(*sQ)[TQ][KCP] =
+        reinterpret_cast<uint32_t(*)[TQ][KCP]>(smem_raw + 2 * PL_TR * KCP * sizeof(uint32_t));
+    TopkSmem<TQ> *tk = reinterpret_cast<TopkSmem<TQ> *>(smem_raw + 2 * (PL_TR + TQ) * KCP * sizeof(uint32_t));
 
     const int tid = threadIdx.x;
     const int lane = tid & 31;
@@ -143,8 +148,8 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
     const uint64_t cut0 = initial_cut(args.threshold);
 
     if (EPI == EPI_TOPK) {
-        for (int i = tid; i < PL_TQ * FASTID_MAX_K; i += PL_THREADS) (&tk->list[0][0])[i] = KEY_EMPTY;
-        for (int i = tid; i < PL_TQ; i += PL_THREADS) {
+        for (int i = tid; i < TQ * FASTID_MAX_K; i += PL_THREADS) (&tk->list[0][0])[i] = KEY_EMPTY;
+        for (int i = tid; i < TQ; i += PL_THREADS) {
             tk->cut[i] = cut0;
             tk->cnt[i] = 0;
         }
@@ -152,8 +157,8 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
         __syncthreads();
     }
 
-    // Loader mapping: each stage is 128 rows x 16 words per operand = 512
-    // 16-byte chunks; 256 threads copy 2 chunks of R and 2 of Q.
+    // Loader mapping: each stage is 128 (R) and TQ (Q) rows x 16 words, four
+    // 16-byte chunks a row; 256 threads copy 2 chunks of R and up to 2 of Q.
     // Stage s of a unit goes to buffer (g + s) & 1, g counting the stages of
     // the CTA's earlier units, so that the next unit's first stage can be
     // copied into the free buffer during this unit's last stage and epilogue.
@@ -163,7 +168,8 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
             int chunk = tid + t * PL_THREADS;  // 0..511
             int row = chunk >> 2, part = chunk & 3;
             cp_async16(&sR[st][row][part * 4], gR_ + row * args.ld32 + kc * PL_KC + part * 4);
-            cp_async16(&sQ[st][row][part * 4], gQ_ + row * args.ld32 + kc * PL_KC + part * 4);
+            if (JQ >= 8 || chunk < 4 * TQ)
+                cp_async16(&sQ[st][row][part * 4], gQ_ + row * args.ld32 + kc * PL_KC + part * 4);
         }
         cp_async_commit();
     };
@@ -175,19 +181,19 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
         const int64_t qt = u / P.n_rt;
         const int64_t rt = u - qt * P.n_rt;
         const int64_t r0 = rt * PL_TR;
-        const int64_t q0 = qt * PL_TQ;
+        const int64_t q0 = qt * TQ;
 
         if (EPI == EPI_TOPK && qt != qt_prev) {
             if (qt_prev >= 0) {
                 // flush the finished segment's lists
-                uint64_t *dst = args.partial + ((c * P.max_seg + seg) * PL_TQ) * (int64_t)args.k;
-                for (int i = tid; i < PL_TQ * args.k; i += PL_THREADS) {
+                uint64_t *dst = args.partial + ((c * P.max_seg + seg) * TQ) * (int64_t)args.k;
+                for (int i = tid; i < TQ * args.k; i += PL_THREADS) {
                     int qq = i / args.k, s = i - qq * args.k;
                     dst[i] = tk->list[qq][s];
                 }
                 __syncthreads();
-                for (int i = tid; i < PL_TQ * FASTID_MAX_K; i += PL_THREADS) (&tk->list[0][0])[i] = KEY_EMPTY;
-                for (int i = tid; i < PL_TQ; i += PL_THREADS) tk->cut[i] = cut0;
+                for (int i = tid; i < TQ * FASTID_MAX_K; i += PL_THREADS) (&tk->list[0][0])[i] = KEY_EMPTY;
+                for (int i = tid; i < TQ; i += PL_THREADS) tk->cut[i] = cut0;
                 __syncthreads();
                 ++seg;
             }
@@ -197,11 +203,11 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
         const uint32_t *gR = args.refs32 + r0 * args.ld32;
         const uint32_t *gQ = args.q32 + q0 * args.ld32;
 
-        uint32_t acc[8][8];
+        uint32_t acc[8][JQ];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = 0;
+            for (int j = 0; j < JQ; ++j) acc[i][j] = 0;
 
         if (!staged) issue_stage(g & 1, gR, gQ, 0);
         for (int kc = 0; kc < args.n_kc; ++kc) {
@@ -212,7 +218,7 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
             } else if (u + 1 < u_end) {  // the next unit's first stage
                 const int64_t qn = (u + 1) / P.n_rt;
                 const int64_t rn = (u + 1) - qn * P.n_rt;
-                issue_stage(st ^ 1, args.refs32 + rn * PL_TR * args.ld32, args.q32 + qn * PL_TQ * args.ld32, 0);
+                issue_stage(st ^ 1, args.refs32 + rn * PL_TR * args.ld32, args.q32 + qn * TQ * args.ld32, 0);
                 cp_async_wait<1>();
             } else {
                 cp_async_wait<0>();
@@ -222,10 +228,10 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
 #pragma unroll
             for (int kk = 0; kk < PL_KC; kk += 8) {
 #pragma unroll
-                for (int jh = 0; jh < 8; jh += 4) {  // four query columns at a time
-                    uint4 qa[4], qb[4];
+                for (int jh = 0; jh < JQ; jh += JC) {  // (at most) four query columns at a time
+                    uint4 qa[JC], qb[JC];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
+                    for (int j = 0; j < JC; ++j) {
                         qa[j] = *reinterpret_cast<const uint4 *>(&sQ[st][tq + 16 * (jh + j)][kk]);
                         qb[j] = *reinterpret_cast<const uint4 *>(&sQ[st][tq + 16 * (jh + j)][kk + 4]);
                     }
@@ -235,7 +241,7 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
                         const uint4 ra = lds128_once(&sR[st][tr + 16 * i][kk]);
                         const uint4 rb = lds128_once(&sR[st][tr + 16 * i][kk + 4]);
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
+                        for (int j = 0; j < JC; ++j)
                             acc[i][jh + j] = and_popc8(ra, rb, qa[j], qb[j], acc[i][jh + j], args.two);
                     }
                 }
@@ -254,10 +260,10 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
             rvalid[i] = r < args.n_refs;
             nr[i] = __ldg(args.ref_norms + r0 + tr + 16 * i);  // padded rows exist (norm 0)
         }
-        uint32_t sc[8][8];
-        bool qvalid[8];
+        uint32_t sc[8][JQ];
+        bool qvalid[JQ];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < JQ; ++j) {
             int64_t q = q0 + tq + 16 * j;
             qvalid[j] = q < args.n_q;
             QueryCoef cf = args.coef[q];  // padded rows exist
@@ -267,7 +273,7 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
 
         if (EPI == EPI_SCORES16 || EPI == EPI_SCORES32) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
+            for (int j = 0; j < JQ; ++j) {
                 if (!qvalid[j]) continue;
                 int64_t q = q0 + tq + 16 * j;
 #pragma unroll
@@ -283,12 +289,12 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
         } else if (EPI == EPI_HITS) {
             bool any = false;
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
+            for (int j = 0; j < JQ; ++j)
 #pragma unroll
                 for (int i = 0; i < 8; ++i) any |= qvalid[j] && rvalid[i] && sc[i][j] <= args.threshold;
             if (__any_sync(0xffffffffu, any)) {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
+                for (int j = 0; j < JQ; ++j) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         bool pred = qvalid[j] && rvalid[i] && sc[i][j] <= args.threshold;
@@ -310,17 +316,17 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
                 }
             }
         } else {  // EPI_TOPK
-            uint64_t done = 0;  // bit i*8+j: element already staged or rejected
+            uint64_t done = 0;  // bit i*JQ+j: element already staged or rejected
             int pass = 0;
             while (true) {
                 bool staged_any = false;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
+                for (int j = 0; j < JQ; ++j) {
                     const int ql = tq + 16 * j;
                     const uint64_t cut = tk->cut[ql];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
-                        const uint64_t bit = 1ull << (i * 8 + j);
+                        const uint64_t bit = 1ull << (i * JQ + j);
                         if (done & bit) continue;
                         const uint64_t key = make_key(sc[i][j], (uint32_t)(r0 + tr + 16 * i));
                         if (!(qvalid[j] && rvalid[i]) || key >= cut) {
@@ -341,7 +347,7 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
                 if (!__syncthreads_or(staged_any)) break;
                 if (tid == 0) tk->ovf[(pass + 1) & 1] = 0;
                 // merge staged candidates, one warp per query
-                for (int ql = warp; ql < PL_TQ; ql += NWARPS) {
+                for (int ql = warp; ql < TQ; ql += NWARPS) {
                     int cnt = tk->cnt[ql];
                     if (cnt == 0) continue;
                     if (cnt > STG) cnt = STG;
@@ -368,41 +374,71 @@ __global__ void __launch_bounds__(PL_THREADS, 2) plain_kernel(const PlainArgs ar
     }
 
     if (EPI == EPI_TOPK && qt_prev >= 0) {
-        uint64_t *dst = args.partial + ((c * P.max_seg + seg) * PL_TQ) * (int64_t)args.k;
-        for (int i = tid; i < PL_TQ * args.k; i += PL_THREADS) {
+        uint64_t *dst = args.partial + ((c * P.max_seg + seg) * TQ) * (int64_t)args.k;
+        for (int i = tid; i < TQ * args.k; i += PL_THREADS) {
             int qq = i / args.k, s = i - qq * args.k;
             dst[i] = tk->list[qq][s];
         }
     }
 }
 
-size_t plain_smem(int epi) {
-    size_t base = 2 * (size_t)(PL_TR + PL_TQ) * KCP * sizeof(uint32_t);
-    if (epi == EPI_TOPK) base += sizeof(TopkSmem);
+size_t plain_smem(int epi, int tq) {
+    size_t base = 2 * (size_t)(PL_TR + tq) * KCP * sizeof(uint32_t);
+    if (epi == EPI_TOPK)
+        base += tq == 128  ? sizeof(TopkSmem<128>)
+                : tq == 64 ? sizeof(TopkSmem<64>)
+                : tq == 32 ? sizeof(TopkSmem<32>)
+                           : sizeof(TopkSmem<16>);
     return base;
 }
 
+typedef void (*PlainFn)(const PlainArgs);
+
 template <int EPI>
-const void *plain_fn() {
-    return reinterpret_cast<const void *>(&plain_kernel<EPI>);
+PlainFn plain_fn_by_tile(int tq) {
+    switch (tq) {
+        case 16: return plain_kernel<EPI, 1>;
+        case 32: return plain_kernel<EPI, 2>;
+        case 64: return plain_kernel<EPI, 4>;
+        default: return plain_kernel<EPI, 8>;
+    }
 }
 
-const void *plain_fn_by_epi(int epi) {
+PlainFn plain_fn(int epi, int tq) {
     switch (epi) {
-        case EPI_SCORES16: return plain_fn<EPI_SCORES16>();
-        case EPI_SCORES32: return plain_fn<EPI_SCORES32>();
-        case EPI_HITS: return plain_fn<EPI_HITS>();
-        default: return plain_fn<EPI_TOPK>();
+        case EPI_SCORES16: return plain_fn_by_tile<EPI_SCORES16>(tq);
+        case EPI_SCORES32: return plain_fn_by_tile<EPI_SCORES32>(tq);
+        case EPI_HITS: return plain_fn_by_tile<EPI_HITS>(tq);
+        default: return plain_fn_by_tile<EPI_TOPK>(tq);
     }
 }
 
 }  // namespace
 
-int plain_grid_target(int epi, int device) {
+int plain_tile_q(int64_t n_q) {
+    // Padded queries, weighted by the lower tiles' cost a query (more
+    // shared-memory reads of the references for each).  Measured with
+    // fastid_topk_noalloc on 1M references at N = 2048, all against a tile of
+    // 128: 16 queries 1630 -> 287 us (tile 16), 32 1660 -> 485 (32), 64 1775 ->
+    // 895 (64), 130 3290 -> 2010 (five of 32).  Only calls of up to 1024 queries: above, 128 pads little, and the
+    // scratch a call needs stays what it was.
+    if (n_q > 1024) return 128;
+    constexpr int tile[] = {128, 64, 32, 16};
+    constexpr double cost[] = {1.0, 1.02, 1.06, 1.15};
+    int best = 0;
+    double least = 0.0;
+    for (int i = 0; i < 4; ++i) {
+        const double c = cost[i] * (double)((n_q + tile[i] - 1) / tile[i] * tile[i]);
+        if (i == 0 || c < least) best = i, least = c;
+    }
+    return tile[best];
+}
+
+int plain_grid_target(int epi, int tq, int device) {
     int sms = 0, occ = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    const void *fn = plain_fn_by_epi(epi);
-    size_t smem = plain_smem(epi);
+    const void *fn = reinterpret_cast<const void *>(plain_fn(epi, tq));
+    size_t smem = plain_smem(epi, tq);
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, PL_THREADS, smem);
     if (occ < 1) occ = 1;
@@ -438,16 +474,12 @@ cudaError_t launch_plain(int epi, const uint32_t *refs32, const uint32_t *ref_no
     a.partial = partial;
     a.part = part;
     a.status = status;
-    size_t smem = plain_smem(epi);
-    const void *fn = plain_fn_by_epi(epi);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = plain_smem(epi, part.tile_q);
+    const PlainFn fn = plain_fn(epi, part.tile_q);
+    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
-    switch (epi) {
-        case EPI_SCORES16: plain_kernel<EPI_SCORES16><<<part.grid, PL_THREADS, smem, s>>>(a); break;
-        case EPI_SCORES32: plain_kernel<EPI_SCORES32><<<part.grid, PL_THREADS, smem, s>>>(a); break;
-        case EPI_HITS: plain_kernel<EPI_HITS><<<part.grid, PL_THREADS, smem, s>>>(a); break;
-        default: plain_kernel<EPI_TOPK><<<part.grid, PL_THREADS, smem, s>>>(a); break;
-    }
+    fn<<<part.grid, PL_THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
 

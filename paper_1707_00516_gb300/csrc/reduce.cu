@@ -51,7 +51,7 @@ __device__ int64_t cta_of(const Partition &P, int64_t u) {
 }
 
 // Plain launches, W warps per query: merge the sorted k-lists of every segment
-// that covered the query's tile.  Segment lists are laid out [slot][PL_TQ][k]
+// that covered the query's tile.  Segment lists are laid out [slot][tile_q][k]
 // with slot = cta * max_seg + (segment index within the CTA).
 __global__ void topk_merge_kernel(const uint64_t *__restrict__ partial, Partition P, int64_t n_q, int32_t k, int W,
                                   uint32_t *__restrict__ out_scores, int64_t *__restrict__ out_idx) {
@@ -61,8 +61,8 @@ __global__ void topk_merge_kernel(const uint64_t *__restrict__ partial, Partitio
     const int64_t q = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) / W;
     int64_t ql = 0, c_lo = 0, c_hi = -1, seg_lo = 0;
     if (q < n_q) {
-        const int64_t qt = q / PL_TQ;
-        ql = q - qt * PL_TQ;
+        const int64_t qt = q / P.tile_q;
+        ql = q - qt * P.tile_q;
         c_lo = cta_of(P, qt * P.n_rt);
         c_hi = cta_of(P, qt * P.n_rt + P.n_rt - 1);
         seg_lo = qt - part_begin(P, c_lo) / P.n_rt;
@@ -70,7 +70,7 @@ __global__ void topk_merge_kernel(const uint64_t *__restrict__ partial, Partitio
     // (only the first CTA can have had an earlier tile: every other one starts inside this tile, segment 0)
     const uint64_t acc = merge_lists((int)(c_hi - c_lo + 1), W, k, lane, sm, [&](int i) {
         const int64_t slot = (c_lo + i) * P.max_seg + (i == 0 ? seg_lo : 0);
-        return lane < k ? partial[(slot * PL_TQ + ql) * k + lane] : KEY_EMPTY;
+        return lane < k ? partial[(slot * P.tile_q + ql) * k + lane] : KEY_EMPTY;
     });
     if (q < n_q && (warp & (W - 1)) == 0 && lane < k) {
         out_scores[q * k + lane] = acc == KEY_EMPTY ? 0xFFFFFFFFu : (uint32_t)(acc >> 32);
@@ -433,7 +433,7 @@ static int merge_block_warps(int W) { return W > 8 ? W : 8; }
 cudaError_t launch_topk_merge(const uint64_t *partial, const Partition &part, int64_t n_q, int32_t k,
                               uint32_t *out_scores, int64_t *out_idx, cudaStream_t s) {
     if (n_q == 0) return cudaSuccess;
-    const int64_t n_qt = (n_q + PL_TQ - 1) / PL_TQ;
+    const int64_t n_qt = part.n_qt;
     const int W = merge_warps(n_q, (part.grid + n_qt - 1) / n_qt + 1), per = merge_block_warps(W) / W;
     topk_merge_kernel<<<(unsigned)((n_q + per - 1) / per), per * W * 32, 0, s>>>(partial, part, n_q, k, W, out_scores,
                                                                                 out_idx);
