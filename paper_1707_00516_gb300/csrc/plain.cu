@@ -420,7 +420,7 @@ int plain_tile_q(int64_t n_q) {
     // shared-memory reads of the references for each).  Measured with
     // fastid_topk_noalloc on 1M references at N = 2048, all against a tile of
     // 128: 16 queries 1630 -> 287 us (tile 16), 32 1660 -> 485 (32), 64 1775 ->
-    // 895 (64), 130 3290 -> 2010 (five of 32).  Only calls of up to 1024 queries: above, 128 pads little, and the
+    // 895 (64), 130 3290 -> 2010 (nine of 16).  Only calls of up to 1024 queries: above, 128 pads little, and the
     // scratch a call needs stays what it was.
     if (n_q > 1024) return 128;
     constexpr int tile[] = {128, 64, 32, 16};

@@ -8,6 +8,8 @@ top-k in the library's kernels and copies the result back.
 """
 from __future__ import annotations
 
+import math
+
 import numpy as np
 import torch
 
@@ -27,6 +29,7 @@ class Searcher:
         B.fastid_set_form(self.ctx, form)
         self._pinned: dict[str, torch.Tensor] = {}
         self._devbuf: dict[str, torch.Tensor] = {}
+        self._devview: dict[str, tuple] = {}  # a buffer's last shape and its view
 
     # ---- database ------------------------------------------------------
     def load_refs_packed(self, packed: torch.Tensor, n_loci: int, flags: int = 0) -> B.RefDB:
@@ -54,9 +57,9 @@ class Searcher:
         n_src = src_alleles.shape[0]
         n_q = offsets.numel() - 1
         w = words64(n_loci)
-        src_packed = self._buf("src_packed", (max(n_src, 1), w), torch.int64)[:n_src]
+        src_packed = self._buf("src_packed", (n_src, w), torch.int64)
         B.fastid_pack(self.ctx, src_alleles, n_loci, src_packed)
-        q = self._buf("queries", (max(n_q, 1), w), torch.int64)[:n_q]
+        q = self._buf("queries", (n_q, w), torch.int64)
         B.fastid_mix(self.ctx, src_packed, w, offsets, q)
         return q
 
@@ -114,12 +117,18 @@ class Searcher:
 
     # ---- host in, host out ---------------------------------------------
     def _buf(self, name, shape, dtype):
+        shape = tuple(shape)
+        last = self._devview.get(name)
+        if last is not None and last[0] == shape and last[1] == dtype:
+            return last[2]
         t = self._devbuf.get(name)
-        n = int(np.prod(shape))
+        n = math.prod(shape)
         if t is None or t.numel() < n or t.dtype != dtype:
-            t = torch.empty(n, dtype=dtype, device=self.device)
+            t = torch.empty(max(n, 1), dtype=dtype, device=self.device)
             self._devbuf[name] = t
-        return t[:n].view(shape)
+        v = t[:n].view(shape)
+        self._devview[name] = (shape, dtype, v)
+        return v
 
     def _pin(self, name, arr: np.ndarray) -> torch.Tensor:
         t = self._pinned.get(name)
