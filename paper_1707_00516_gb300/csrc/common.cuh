@@ -179,6 +179,7 @@ struct TcLaunch {
     unsigned long long *hit_count;
     uint64_t *partial;  // EPI_TOPK: [n_slots][k][128]
     uint32_t *status;
+    int32_t dependent;  // the merge may be launched beside the compare kernel's end (see launch_dependent)
     // Panel-entry counters, one per position of the panel order (zero before
     // the launch), or nullptr: see the rendezvous in the tensor kernel.
     unsigned int *arrive;
@@ -192,6 +193,26 @@ struct TcLaunch {
 int32_t make_tensor_schedule(int n, const int64_t *n_qq, const int64_t *n_rt, const int64_t *tile_bytes,
                              int32_t G, int32_t ctas_per_group, TcSched *sched, int32_t *order,
                              int32_t *n_slots);
+
+#ifdef __CUDACC__
+// Launch of a kernel that begins beside the end of the one before it on the
+// stream (programmatic dependent launch) and calls griddepcontrol.wait before
+// it touches anything that one writes.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#endif
 
 // Top-k keys: (score << 32) | ref, so that ordering keys orders by score then
 // by reference index.  An empty slot holds KEY_EMPTY.

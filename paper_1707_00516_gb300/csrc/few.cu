@@ -79,7 +79,10 @@ constexpr uint32_t FQ_SF_COL = 448;  // unit scale factors, 64 columns
 constexpr int FQ_QUEUE = 32;         // ring entries a query: one a lane when merged
 constexpr int FQ_MERGE_MIN = 8;      // rings of this many entries are merged before shorter ones
 constexpr int FQ_SLICES_MAX = 256;   // slices whose published scores a warp looks through
-constexpr int FQ_SAMPLE_MAX = 1024;  // sampled references of the seed kernel
+constexpr int FQ_SEED_WARPS = 32;    // seed kernel: one encodes, the others score FQ_SEED_ROWS references each
+constexpr int FQ_SEED_ROWS = 8;
+constexpr int FQ_SAMPLE_ROUND = (FQ_SEED_WARPS - 1) * FQ_SEED_ROWS;
+constexpr int FQ_SAMPLE_MAX = 4 * FQ_SAMPLE_ROUND;
 
 struct FewArgs {
     int64_t n_refs;
@@ -274,6 +277,8 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
         for (int c = 0; c < (int)FQ_A_COL; c += 16) tmem_fill16(lanes + c, 0u);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
+    // (everything up to here ran beside the seed kernel)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const float INF = __int_as_float(0x7f800000);
     const float t1 = A.threshold == 0xFFFFFFFFu ? INF : (float)A.threshold + 1.0f;
     if (tid < FQ_N) {
@@ -479,7 +484,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
                 union_q += A.slices;  // fewer slices than queries: several in turn
                 if (union_q >= A.n_q) union_q = first_q;
             }
-            __nanosleep(1000);
+            __nanosleep(300);
         }
         __syncwarp();
         // The lists: slot = CTA, [k][128].
@@ -612,6 +617,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
         }
     }
 
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the merge, which waits for these results
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -619,25 +625,32 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-// Query operand and starting cut, a block of 32 warps a row: warp 0 encodes
-// the row (the inverses of the expansion, see the top) and its constant; all score a strided sample of the references
-// against the query, and the k-th smallest of those bounds every result entry
-// of the query (there are k references no worse).
-__global__ void __launch_bounds__(1024) few_seed_kernel(const uint64_t *__restrict__ q, int64_t ld_q, int64_t n_q,
-                                                        int32_t n_words, int32_t n_loci,
-                                                        const uint8_t *__restrict__ modes, int32_t kbytes,
-                                                        uint8_t *__restrict__ out, float *__restrict__ qconst,
-                                                        const SharedCut cut,
-                                                        const uint64_t *__restrict__ refs, int64_t ld_r,
-                                                        int64_t n_refs, int sample, int k, int32_t *__restrict__ pub,
-                                                        int32_t slices) {
+// Query operand and starting cut, a block a row: warp 0 encodes the row (the
+// inverses of the expansion, see the top) and its constant; the others score
+// a strided sample of the references against the query, and the k-th smallest
+// of those bounds every result entry of the query (there are k references no
+// worse).  The kernel is a chain of latencies (1024 samples for every call
+// and a block barrier in each bisection step: 16 us of a 38 us call), so a
+// warp loads 8 references at once, few calls take a second round, one warp
+// selects alone, and the compare kernel sets itself up meanwhile.
+__global__ void __launch_bounds__(FQ_SEED_WARPS * 32)
+    few_seed_kernel(const uint64_t *__restrict__ q, int64_t ld_q, int64_t n_q, int32_t n_words, int32_t n_loci,
+                    const uint8_t *__restrict__ modes, int32_t kbytes, uint8_t *__restrict__ out,
+                    float *__restrict__ qconst, const SharedCut cut, const uint64_t *__restrict__ refs, int64_t stride,
+                    int sample, int k, int32_t *__restrict__ pub, int32_t slices) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the compare kernel waits for this one's results)
     __shared__ uint32_t sc[FQ_SAMPLE_MAX];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t r = blockIdx.x;
     const bool valid = r < n_q;
     const uint64_t *qr = q + r * ld_q;
     const bool mis = valid && modes[r] == FASTID_MODE_MISMATCH;
+    int32_t best = NET_EMPTY;
     if (warp == 0) {
+        if (valid && cut.run_s) {
+            const int64_t last = r * cut.k + cut.k - 1;
+            if (cut.run_i[last] >= 0 && cut.run_s[last] <= (uint32_t)FASTID_MAX_LOCI) best = (int32_t)cut.run_s[last];
+        }
         uint32_t pc = 0;
         int32_t a3 = 0;  // sum of a over the j = 3 loci
         for (int32_t c = lane; c < kbytes / 16; c += 32) {
@@ -663,54 +676,46 @@ __global__ void __launch_bounds__(1024) few_seed_kernel(const uint64_t *__restri
         pc = __reduce_add_sync(0xffffffffu, pc);
         a3 = __reduce_add_sync(0xffffffffu, a3);
         if (lane == 0) qconst[r] = (mis ? (float)pc : 0.f) + 0.5f * (float)a3;
-    }
-    for (int i = threadIdx.x; i < slices; i += blockDim.x) pub[r * slices + i] = NET_EMPTY;
-    if (!valid) {
-        if (threadIdx.x == 0) cut.out[r] = NET_EMPTY;
-        return;
-    }
-    int32_t best = NET_EMPTY;
-    if (sample >= k && sample > 0) {
-        const int64_t stride = n_refs / sample * ld_r;
-        for (int i0 = warp; i0 < sample; i0 += 32 * 8) {
-            uint32_t pc[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+        for (int i = lane; i < slices; i += 32) pub[r * slices + i] = NET_EMPTY;
+    } else if (valid) {
+        for (int i0 = (warp - 1) * FQ_SEED_ROWS; i0 < sample; i0 += FQ_SAMPLE_ROUND) {
+            uint32_t pc[FQ_SEED_ROWS] = {};
             for (int32_t w = lane; w < n_words; w += 32) {
+                uint64_t rw[FQ_SEED_ROWS];
                 const uint64_t qw = qr[w];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + u * 32;
-                    if (i < sample) {
-                        const uint64_t rw = refs[i * stride + w];
-                        pc[u] += __popcll(mis ? rw ^ qw : rw & ~qw);
-                    }
-                }
+                for (int u = 0; u < FQ_SEED_ROWS; ++u) rw[u] = i0 + u < sample ? refs[(i0 + u) * stride + w] : 0ull;
+#pragma unroll
+                for (int u = 0; u < FQ_SEED_ROWS; ++u) pc[u] += __popcll(mis ? rw[u] ^ qw : rw[u] & ~qw);
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < FQ_SEED_ROWS; ++u) {
                 const uint32_t s = __reduce_add_sync(0xffffffffu, pc[u]);
-                if (lane == 0 && i0 + u * 32 < sample) sc[i0 + u * 32] = s;
+                if (lane == 0 && i0 + u < sample) sc[i0 + u] = s;
             }
         }
-        __syncthreads();
-        const uint32_t mine = (int)threadIdx.x < sample ? sc[threadIdx.x] : 0xFFFFFFFFu;
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    if (valid && sample >= k) {
+        constexpr int V = FQ_SAMPLE_MAX / 32;
+        uint32_t v[V];
+#pragma unroll
+        for (int u = 0; u < V; ++u) v[u] = u * 32 + lane < sample ? sc[u * 32 + lane] : 0xFFFFFFFFu;
         uint32_t lo = 0, hi = (uint32_t)n_loci;
         while (lo < hi) {  // the smallest value with k samples at or below it
             const uint32_t mid = (lo + hi) >> 1;
-            if (__syncthreads_count(mine <= mid) >= k)
+            uint32_t n = 0;
+#pragma unroll
+            for (int u = 0; u < V; ++u) n += v[u] <= mid;
+            if (__reduce_add_sync(0xffffffffu, n) >= (uint32_t)k)
                 hi = mid;
             else
                 lo = mid + 1;
         }
-        best = (int32_t)lo;
+        best = min(best, (int32_t)lo);
     }
-    if (threadIdx.x == 0) {
-        if (cut.run_s) {
-            const int64_t last = r * cut.k + cut.k - 1;
-            if (cut.run_i[last] >= 0 && cut.run_s[last] <= (uint32_t)FASTID_MAX_LOCI)
-                best = min(best, (int32_t)cut.run_s[last]);
-        }
-        cut.out[r] = best;
-    }
+    if (lane == 0) cut.out[r] = best;
 }
 
 constexpr uint32_t FQ_SMEM_MAX = 227u * 1024u;
@@ -729,11 +734,18 @@ bool few_shape(int64_t n_q, int32_t n_loci, int32_t k, FewShape *S) {
 }
 
 cudaError_t launch_few_seed(const FewLaunch &L, const FewShape &S, cudaStream_t s) {
-    // as many samples as a sixteenth of the references, at most FQ_SAMPLE_MAX
-    const int sample = (int)std::min<int64_t>(FQ_SAMPLE_MAX, L.n_refs / 16);
-    few_seed_kernel<<<(unsigned)S.ncols, 1024, 0, s>>>(
-        L.q, L.ld_q, L.n_q, L.n_words, L.n_loci, L.modes, S.n_kb * 128, L.operand, L.qconst, L.cut, L.packed,
-        L.ld64, L.n_refs, sample, L.k, L.pub, L.slices);
+    // At most a sixteenth of the references.  With up to 8 queries the seeds
+    // are on the call's critical path and one round is enough (one query over
+    // 2M x 2048: 132.7 us with one round, 141.9 with four; over 200000 x 1024
+    // the same); with more the first tiles' candidates cost more than the
+    // rounds (48 queries, top 32 of 200000 x 1024: 151 us with one, 115 with
+    // four, 97 with eight, but 16 queries over 50000 40.7, 41.5 and 45.8).
+    const int rounds = L.n_q <= 8 ? 1 : FQ_SAMPLE_MAX / FQ_SAMPLE_ROUND;
+    const int sample = (int)std::min<int64_t>(rounds * FQ_SAMPLE_ROUND, L.n_refs / 16);
+    const int64_t stride = sample > 0 ? L.n_refs / sample * L.ld64 : 0;
+    few_seed_kernel<<<(unsigned)S.ncols, FQ_SEED_WARPS * 32, 0, s>>>(
+        L.q, L.ld_q, L.n_q, L.n_words, L.n_loci, L.modes, S.n_kb * 128, L.operand, L.qconst, L.cut, L.packed, stride,
+        sample, L.k, L.pub, L.slices);
     return cudaGetLastError();
 }
 
@@ -763,8 +775,7 @@ cudaError_t launch_few(const FewLaunch &L, const FewShape &S, cudaStream_t s) {
     const uint32_t smem = few_smem_bytes(S.ncols, S.n_kb, S.stages, L.k);
     e = cudaFuncSetAttribute(few_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FQ_SMEM_MAX);
     if (e != cudaSuccess) return e;
-    few_kernel<<<(unsigned)L.slices, FQ_THREADS, smem, s>>>(map_q, map_r, a);
-    return cudaGetLastError();
+    return launch_dependent(few_kernel, dim3((unsigned)L.slices), dim3(FQ_THREADS), smem, s, map_q, map_r, a);
 }
 
 }  // namespace fastid

@@ -118,6 +118,7 @@ __global__ void topk_merge_sched_kernel(const uint64_t *__restrict__ partial, co
                                         const MergeJob *__restrict__ jobs, int64_t n_jobs, int W,
                                         uint32_t *__restrict__ out_s, int64_t *__restrict__ out_i) {
     __shared__ uint64_t sm[MERGE_MAX_WARPS][32];
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // (returns at once in an ordinary launch)
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int64_t j = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) / W;
@@ -458,8 +459,11 @@ cudaError_t launch_merge_sched(const uint64_t *partial, const TcLaunch &L, const
     for (int p = 0; p < L.n_panels; ++p)
         n_lists = std::max<int64_t>(n_lists, L.sched[p].b + (L.sched[p].t_groups > 0 ? 1 : 0));
     const int W = merge_warps(n_jobs, n_lists), per = merge_block_warps(W) / W;
-    topk_merge_sched_kernel<<<(unsigned)((n_jobs + per - 1) / per), per * W * 32, 0, s>>>(partial, M, jobs, n_jobs, W,
-                                                                                         out_scores, out_idx);
+    const dim3 grid((unsigned)((n_jobs + per - 1) / per)), block(per * W * 32);
+    if (L.dependent)
+        return launch_dependent(topk_merge_sched_kernel, grid, block, 0, s, partial, M, jobs, n_jobs, W, out_scores,
+                                out_idx);
+    topk_merge_sched_kernel<<<grid, block, 0, s>>>(partial, M, jobs, n_jobs, W, out_scores, out_idx);
     return cudaGetLastError();
 }
 
