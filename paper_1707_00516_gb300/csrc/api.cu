@@ -554,10 +554,12 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
     Carver cv;
     size_t o_a = cv.take<uint8_t>((size_t)n_q_pad * kbytes);
     size_t o_c = cv.take<float>((size_t)n_q_pad);
-    size_t o_g = cv.take<int32_t>(ek == EXTRA_TOPK ? (size_t)n_q_pad : 0);
+    if (ek == EXTRA_TOPK) plan_pub(L, 0, (int32_t)karg);
+    size_t o_g = cv.take<int32_t>(ek == EXTRA_TOPK ? (size_t)n_q_pad * (1 + L.n_pub[0]) : 0);
     *extra_off = cv.take<uint8_t>(extra);
     FASTID_CUDA(ctx, scr.alloc(cv.off));
-    const SharedCut cut{ek == EXTRA_TOPK ? at<int32_t>(scr.p, o_g) : nullptr, run_s, run_i, (int32_t)karg};
+    const SharedCut cut{ek == EXTRA_TOPK ? at<int32_t>(scr.p, o_g) : nullptr, run_s, run_i, (int32_t)karg, n_q_pad,
+                        L.n_pub[0]};
     uint8_t *a = at<uint8_t>(scr.p, o_a);
     float *qconst = at<float>(scr.p, o_c);
     // spread the input queries over every tile of the operand (see
@@ -582,6 +584,7 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
     L.kpad[0] = kbytes;
     L.qconst[0] = qconst;
     L.gcut[0] = cut.out;
+    L.gcut_ld[0] = n_q_pad;
     L.qspread[0] = (int32_t)spread;
     L.status = ctx->dev_status;
     return FASTID_OK;

@@ -77,7 +77,9 @@ struct PrepJob {
     const uint8_t *mode;   // its mode byte
     uint8_t *dst;          // operand row [kpad bytes]: e4m3, or e2m1 when f4
     float *qc;             // its c_q
-    int32_t *gc;           // its shared cut (see TcLaunch::gcut)
+    int32_t *gc;           // its shared cut, and
+    int64_t gc_ld;         // n_pub published bounds after it at this stride (see TcLaunch::gcut)
+    int32_t n_pub;
     int32_t n_words;
     int32_t n_loci;
     int32_t kpad;          // operand row bytes
@@ -158,7 +160,15 @@ struct TcLaunch {
     // list fills (set by the encoders to none, or to a running list's k-th).
     // Candidates of a higher score are dropped, those of the same score are not
     // (their reference may be lower).
+    // Rows 1 .. n_pub of [1 + n_pub][gcut_ld]: the pub_rank-th best score of each
+    // reference slice's list (the tail's slice last), published as it improves.
+    // pub_need slices at or below x hold k references at or below x, so the
+    // pub_need-th smallest of any group of slices bounds every result entry
+    // (see plan_pub and the epilogue).
     int32_t *gcut[TC_MAXP];
+    int64_t gcut_ld[TC_MAXP];  // operand rows
+    int32_t n_pub[TC_MAXP];    // 0: one slice, or k = 1 (the shared cut says as much)
+    int32_t pub_rank[TC_MAXP], pub_need[TC_MAXP];
     // Query spreading (see spread_row_to_query): the panel's operand tiles
     // (0 or 1: operand row r holds input query r).  Batched plans spread each
     // panel's queries in batch order and give the merge their rows.
@@ -193,6 +203,21 @@ struct TcLaunch {
 int32_t make_tensor_schedule(int n, const int64_t *n_qq, const int64_t *n_rt, const int64_t *tile_bytes,
                              int32_t G, int32_t ctas_per_group, TcSched *sched, int32_t *order,
                              int32_t *n_slots);
+
+// Published bounds of a top-k launch's panel (TcLaunch::n_pub, pub_rank,
+// pub_need) for its schedule: n_pub rows, groups of up to TC_UNION slices.
+constexpr int TC_UNION = 16;
+inline void plan_pub(TcLaunch &L, int p, int32_t k) {
+    const TcSched &sc = L.sched[p];
+    const int32_t n = sc.b + (sc.t_groups > 0 ? 1 : 0);
+    L.n_pub[p] = n >= 2 && k >= 2 ? n : 0;
+    const int32_t m = n < TC_UNION ? n : TC_UNION;
+    // five slices of eight have to reach the bound: all of them is the slowest
+    // slice's, one of them its k-th, which the shared cut holds already
+    const int32_t want = (5 * m + 7) / 8 < 2 ? 2 : (5 * m + 7) / 8;
+    L.pub_rank[p] = (k + want - 1) / want;
+    L.pub_need[p] = (k + L.pub_rank[p] - 1) / L.pub_rank[p];
+}
 
 #ifdef __CUDACC__
 // Launch of a kernel that begins beside the end of the one before it on the
@@ -277,6 +302,8 @@ struct SharedCut {
     const uint32_t *run_s;  // [n_q][k], or nullptr
     const int64_t *run_i;
     int32_t k;
+    int64_t ld;     // operand rows: n_pub rows of published bounds, none yet, follow out's
+    int32_t n_pub;
 };
 // FP8 reference operand [n_rows][kpad] from packed rows (n_src rows of n_words
 // words exist at stride ld64; zero elsewhere), on at most max_blocks CTAs.

@@ -172,7 +172,9 @@ fastid_status fastid_plan_create(fastid_ctx *ctx, const fastid_refdb *const *dbs
     for (int p = 0; p < n_panels; ++p) {
         o_a[p] = take((size_t)rows_pad[p] * kbytes(p));
         o_qc[p] = take((size_t)rows_pad[p] * sizeof(float));
-        o_gc[p] = take((size_t)rows_pad[p] * sizeof(int32_t));
+        plan_pub(L, p, k);
+        L.gcut_ld[p] = rows_pad[p];
+        o_gc[p] = take((size_t)rows_pad[p] * (1 + L.n_pub[p]) * sizeof(int32_t));
         n_prep += rows_pad[p];
     }
     const size_t o_prep = take((size_t)n_prep * sizeof(PrepJob));
@@ -207,6 +209,8 @@ fastid_status fastid_plan_create(fastid_ctx *ctx, const fastid_refdb *const *dbs
                 j.dst = W + o_a[p] + (size_t)r * kbytes(p);
                 j.qc = reinterpret_cast<float *>(W + o_qc[p]) + r;
                 j.gc = reinterpret_cast<int32_t *>(W + o_gc[p]) + r;
+                j.gc_ld = rows_pad[p];
+                j.n_pub = L.n_pub[p];
                 j.n_words = dbs[p]->n_words64;
                 j.n_loci = dbs[p]->n_loci;
                 j.kpad = (int32_t)kbytes(p);

@@ -264,6 +264,10 @@ __device__ __forceinline__ int32_t load_cut(const int32_t *p) {
     return v;
 }
 
+__device__ __forceinline__ void store_cut(int32_t *p, int32_t v) {
+    asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 // Bounded wait that ignores the abort flag: used to drain this CTA's own
 // asynchronous copies and MMAs before it exits.
 __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity, uint32_t *status, uint32_t site) {

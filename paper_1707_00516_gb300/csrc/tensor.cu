@@ -97,7 +97,9 @@ struct PanelDesc {
     int32_t n_kb;         // K stages of 128 operand bytes
     TcSched sc;
     const float *qconst;  // c_q per padded query row
-    int32_t *gcut;        // shared cut per padded query row, or nullptr (see TcLaunch)
+    int32_t *gcut;        // shared cut per padded query row, or nullptr, and the
+    int64_t gcut_ld;      // slices' published bounds (see TcLaunch)
+    int32_t n_pub, pub_rank, pub_need;
     int32_t qspread;      // see spread_row_to_query
 };
 
@@ -232,6 +234,36 @@ __device__ __forceinline__ void queue_insert(const uint32_t *queue, int queued, 
     }
 }
 
+// The need-th smallest of a group's published bounds (see TcLaunch::gcut) for
+// this lane's query row: n values at stride ld, the first TC_UNION of them.
+// A slice's own k-th is the k-th of what that slice has seen; the union's is
+// near the k-th of what all of them have, so with b slices the lists fill with
+// a b-th of the candidates.  Read and sorted (1000 cycles, 16 loads at once)
+// only at the tile after a flush.  Measured, k = 16, no threshold, FP4: 1792
+// queries x 250,000 references, N = 512 399 -> 329 us, N = 2048 424 -> 362;
+// 2048 queries x 2M, N = 2048 2140 -> 2010; 500 x 2M 703 -> 604.
+__device__ __forceinline__ int32_t union_cut(const int32_t *pub, int64_t ld, int n, int need) {
+    int32_t u[TC_UNION];
+#pragma unroll
+    for (int i = 0; i < TC_UNION; ++i) u[i] = i < n ? load_cut(pub + i * ld) : NET_EMPTY;
+#pragma unroll
+    for (int size = 2; size <= TC_UNION; size *= 2)
+#pragma unroll
+        for (int step = size / 2; step > 0; step /= 2)
+#pragma unroll
+            for (int i = 0; i < TC_UNION; ++i) {
+                const int j = i ^ step;
+                if (j <= i) continue;
+                const int32_t lo = min(u[i], u[j]), hi = max(u[i], u[j]);
+                u[i] = (i & size) == 0 ? lo : hi;
+                u[j] = (i & size) == 0 ? hi : lo;
+            }
+    int32_t x = u[0];  // (u ascends)
+#pragma unroll
+    for (int i = 1; i < TC_UNION; ++i) x = max(x, i < need ? u[i] : u[0]);
+    return x;
+}
+
 struct TcSmem {
     uint64_t full[8];
     uint64_t empty[8];
@@ -340,6 +372,7 @@ struct GroupWork {
     int64_t r_lo, r_hi;
     int32_t q_lo, q_hi, chunk;
     int64_t slot;
+    int32_t slice;  // reference slice: y, or b for the tail
 };
 
 // cpg: CTAs per group (2 when paired), rank: this CTA's rank in its group.
@@ -349,6 +382,7 @@ __device__ __forceinline__ GroupWork group_work(const TensorArgs &a, int64_t wg,
     w.q_lo = w.q_hi = 0;
     w.chunk = 1;
     w.slot = 0;
+    w.slice = 0;
     const TcSched &sc = a.panel[p].sc;
     const int64_t grid = (int64_t)sc.a * sc.b;
     if (sc.n_qq <= 0) return w;
@@ -360,6 +394,7 @@ __device__ __forceinline__ GroupWork group_work(const TensorArgs &a, int64_t wg,
         w.q_hi = (int32_t)min((int64_t)sc.n_qq, (x + 1) * sc.tpx);
         w.chunk = sc.chunk;
         w.slot = (int64_t)sc.slot0 + (wg * cpg + rank) * sc.tpx;
+        w.slice = (int32_t)y;
     } else if (wg < grid + sc.t_groups) {
         const int64_t t = wg - grid;
         w.r_lo = sc.r_main;
@@ -368,6 +403,7 @@ __device__ __forceinline__ GroupWork group_work(const TensorArgs &a, int64_t wg,
         w.q_hi = (int32_t)min((int64_t)sc.n_qq, (t + 1) * sc.t_tpx);
         w.chunk = sc.t_chunk;
         w.slot = (int64_t)sc.slot0 + grid * cpg * sc.tpx + (t * cpg + rank) * sc.t_tpx;
+        w.slice = sc.b;
     }
     return w;
 }
@@ -865,10 +901,20 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                         cut = ls[KM - 1] == NET_EMPTY ? cut0 : (float)ls[KM - 1] - cq;
                         if (shared != NET_EMPTY) cut = fminf(cut, (float)(shared + 1) - cq);
                     };
+                    const int32_t n_pub = gc ? P.n_pub : 0;
+                    const int32_t win = min(W.slice / TC_UNION * TC_UNION, max(0, n_pub - TC_UNION));
+                    bool due = false;  // something was published since the last union
                     auto share_cut = [&]() {
                         if (gc && ls[KM - 1] < shared) {
                             shared = ls[KM - 1];
                             atomicMin(gc, shared);
+                        }
+                        if (n_pub > 0) {
+                            int32_t mine = ls[0];  // (ls ascends)
+#pragma unroll
+                            for (int i = 1; i < KM; ++i) mine = max(mine, i < KM - k + P.pub_rank ? ls[i] : ls[0]);
+                            store_cut(gc + (1 + W.slice) * P.gcut_ld, mine);
+                            due = true;
                         }
                     };
                     set_cut();
@@ -896,6 +942,15 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                                 set_cut();
                             }
                             newer = load_cut(gc);
+                        }
+                        if (due) {  // (the same for the whole warp)
+                            due = false;
+                            const int32_t x = union_cut(gc + (1 + win) * P.gcut_ld, P.gcut_ld, n_pub - win, P.pub_need);
+                            if (x < shared) {
+                                shared = x;
+                                atomicMin(gc, x);
+                                set_cut();
+                            }
                         }
                         if (topk && r0 + BN - qbase > TC_QSPAN) {  // the queues' reference window moves on
                             flush();
@@ -1175,6 +1230,9 @@ __device__ __forceinline__ void init_cut(const SharedCut &cut, int64_t r, int64_
     }
     cut.out[r] = c;
 }
+__device__ __forceinline__ void init_pub(int32_t *row, int64_t ld, int32_t n_pub, int lane) {
+    for (int i = lane; i < n_pub; i += 32) row[(1 + i) * ld] = NET_EMPTY;
+}
 
 // Operand row r encodes input query spread_row_to_query(r, spread).
 __global__ void queries_e2m1_kernel(const uint64_t *__restrict__ q, int64_t ld_q, int64_t n_q, int32_t n_words,
@@ -1187,6 +1245,7 @@ __global__ void queries_e2m1_kernel(const uint64_t *__restrict__ q, int64_t ld_q
         const int64_t src = spread_row_to_query(r, spread);
         const bool valid = src < n_q;
         if (cut.out && lane == 0) init_cut(cut, r, src, valid);
+        if (cut.out) init_pub(cut.out + r, cut.ld, cut.n_pub, lane);
         encode_query_row_f4(valid ? q + src * ld_q : nullptr, valid && modes[src] == FASTID_MODE_MISMATCH, n_words,
                             n_loci, kbytes, out + r * (int64_t)kbytes, qconst + r, lane);
     }
@@ -1202,6 +1261,7 @@ __global__ void queries_e4m3_kernel(const uint64_t *__restrict__ q, int64_t ld_q
         const int64_t src = spread_row_to_query(r, spread);
         const bool valid = src < n_q;
         if (cut.out && lane == 0) init_cut(cut, r, src, valid);
+        if (cut.out) init_pub(cut.out + r, cut.ld, cut.n_pub, lane);
         encode_query_row(valid ? q + src * ld_q : nullptr, valid && modes[src] == FASTID_MODE_MISMATCH, n_words,
                          n_loci, kpad, out + r * (int64_t)kpad, qconst + r, lane, one, pk);
     }
@@ -1215,6 +1275,7 @@ __global__ void prep_jobs_kernel(const PrepJob *__restrict__ jobs, int64_t n_job
         const PrepJob jb = jobs[j];
         const bool mis = jb.src != nullptr && *jb.mode == FASTID_MODE_MISMATCH;
         if (lane == 0) *jb.gc = NET_EMPTY;
+        init_pub(jb.gc, jb.gc_ld, jb.n_pub, lane);
         if (jb.f4)
             encode_query_row_f4(jb.src, mis, jb.n_words, jb.n_loci, jb.kpad, jb.dst, jb.qc, lane);
         else
@@ -1418,6 +1479,10 @@ cudaError_t launch_tensor_multi(int bn, const TcLaunch &L, cudaStream_t s) {
         a.panel[p].sc = L.sched[p];
         a.panel[p].qconst = L.qconst[p];
         a.panel[p].gcut = L.gcut[p];
+        a.panel[p].gcut_ld = L.gcut_ld[p];
+        a.panel[p].n_pub = L.n_pub[p];
+        a.panel[p].pub_rank = L.pub_rank[p];
+        a.panel[p].pub_need = L.pub_need[p];
         a.panel[p].qspread = L.qspread[p];
         a.order[p] = L.order[p];
     }
