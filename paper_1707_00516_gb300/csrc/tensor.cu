@@ -84,8 +84,9 @@ struct TcShape {
     static constexpr uint32_t B_BYTES = (uint32_t)(CG2 ? BN / 2 : BN) * TC_BK;
     static constexpr uint32_t TMEM_COLS = BN == 128 ? 256 : 512;
     // beside the ring: transpose buffers, or the candidate queues (QD entries
-    // a query row: 8, or what the fullest ring leaves)
-    static constexpr int QD = CG2 && BN == 256 ? 3 : 8;
+    // a query row: what the fullest rings leave)
+    static constexpr int QD = CG2 && BN == 256 ? 3 : 11;
+    static constexpr int QG = QD < 8 ? 2 : 4;  // columns queued at a time, while QD - QG or fewer are
     static constexpr uint32_t EX_BYTES = SC ? SC_BYTES : (uint32_t)QD * TC_BM * 4;
 };
 
@@ -218,6 +219,44 @@ __device__ __forceinline__ void net_insert(int32_t (&ls)[KM], uint32_t (&lr)[KM]
 // the lower reference first; one that no longer beats the list changes
 // nothing.  The cut is that of the last insertion, so a deeper queue lets more
 // late candidates in: with k = 16 and 8 entries about a fifth more.
+// Adding a column: its entry is stored after the queue's last, and the queue
+// grows by it if it beats the cut -- without a predicate, whose latency is the
+// longest of the steps, and without a branch.  While lists of short streams
+// fill, a third of the 32-column chunks hold a candidate or two, and one warp
+// a scheduler issues all of it; with the chunk's 32 columns unrolled such a
+// chunk took 830 cycles, mostly fetching instructions, which was half of the
+// launch; a short loop over groups of 4 columns, re-read from TMEM, takes 500
+// (FP4, k = 16, no threshold: 1792 queries x 250,000 references N = 512 329 ->
+// 261 us, N = 2048 362 -> 309; 512 x 1M N = 1024 312 -> 260; 2048 x 2M 2010 ->
+// 1936; the FP8 form, MMA-bound at 500 x 2M: 1029 -> 1015).  The score leaves FP32 as the
+// low bits of score + 2^23, which the shift leaves alone in the high bits.
+constexpr uint32_t SCORE_MAGIC = 0x4B000000u;  // 2^23
+
+// The sign of d - cut: an infinite cut keeps its sign, and no d is NaN.
+__device__ __forceinline__ uint32_t queue_step(float d, float cut) {
+    return (__float_as_uint(d - cut) >> 31) * (TC_BM * 4);
+}
+
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float d;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+template <int N, class T>
+__device__ __forceinline__ float group_min(const T *v) {
+    float t[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) t[j] = __builtin_bit_cast(float, v[j]);
+#pragma unroll
+    for (int n = N; n > 1; n = (n + 2) / 3) {
+#pragma unroll
+        for (int j = 0; j < (n + 2) / 3; ++j)
+            t[j] = 3 * j + 2 < n ? min3(t[3 * j], t[3 * j + 1], t[3 * j + 2])
+                                 : 3 * j + 1 < n ? fminf(t[3 * j], t[3 * j + 1]) : t[3 * j];
+    }
+    return t[0];
+}
+
 template <int KM>
 __device__ __forceinline__ void queue_insert(const uint32_t *queue, int queued, int64_t qbase, int32_t (&ls)[KM],
                                              uint32_t (&lr)[KM]) {
@@ -290,7 +329,7 @@ struct TcSmem {
 template <int ESZ>
 __device__ __forceinline__ void store_scores(uint8_t *out, int64_t row_step, int rows, int cols, bool vec,
                                              uint32_t *buf, const uint32_t (&v)[32], float cq, int lane) {
-    constexpr uint32_t MAGIC = 0x4B000000u;  // 2^23
+    constexpr uint32_t MAGIC = SCORE_MAGIC;
     const float cm = cq + __uint_as_float(MAGIC);
     __syncwarp();  // the previous block's reads are done
 #pragma unroll
@@ -975,68 +1014,57 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                                 continue;
                             }
                             // Common case first: nothing in the chunk beats the cut
-                            // (the chunk's minimum, by a tree of fminf).
-                            float mn[16];
+                            // (the minima of its groups of G columns, and theirs).
+                            constexpr int G = S::QG, NG = 32 / G;
+                            float gm[NG];
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) mn[j] = fminf(__uint_as_float(v[j]), __uint_as_float(v[j + 16]));
-#pragma unroll
-                            for (int w = 8; w > 0; w >>= 1)
-#pragma unroll
-                                for (int j = 0; j < w; ++j) mn[j] = fminf(mn[j], mn[j + w]);
-                            if (!__any_sync(0xffffffffu, mn[0] < cut)) continue;
-                            uint32_t m = 0;  // columns of this chunk that pass the filter
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) m |= (uint32_t)(__uint_as_float(v[j]) < cut) << j;
-                            if (rch + 32 > n_refs) m &= rch >= n_refs ? 0u : ((1u << (n_refs - rch)) - 1u);
-                            if (!__any_sync(0xffffffffu, m != 0u)) continue;
+                            for (int g = 0; g < NG; ++g) gm[g] = group_min<G>(v + g * G);
+                            if (!__any_sync(0xffffffffu, group_min<NG>(gm) < cut)) continue;
                             if (args.epi == EPI_HITS) {
-                                append_hits(args, m, taddr + ch * 32, cq, q, rch, lane);
+                                uint32_t m = 0;  // columns of this chunk that pass the filter
+#pragma unroll
+                                for (int j = 0; j < 32; ++j) m |= (uint32_t)(__uint_as_float(v[j]) < cut) << j;
+                                if (rch + 32 > n_refs) m &= rch >= n_refs ? 0u : ((1u << (n_refs - rch)) - 1u);
+                                if (__any_sync(0xffffffffu, m != 0u)) append_hits(args, m, taddr + ch * 32, cq, q, rch, lane);
                                 continue;
                             }
-                            // rare path.  The candidates go to the queues; where they do
-                            // not fit, the queues are inserted first, and a chunk that
-                            // is dense even then (a list still filling) is inserted
-                            // directly, in lock-step and column by column, each column
-                            // re-read from TMEM by the whole warp (the accumulator is
-                            // released only after the tile, below).
-                            if (__any_sync(0xffffffffu, queued + __popc(m) > S::QD)) {
-                                flush();
-                                uint32_t still = 0;
+                            // The candidates go to the queues, a group that some lane
+                            // needs at a time, each re-read from TMEM by the whole
+                            // warp (the accumulator is released only after the tile,
+                            // below): a short loop, which stays in the instruction
+                            // cache where unrolled code over the chunk's registers
+                            // did not (see queue_step).
+                            uint32_t left = 0;
 #pragma unroll
-                                for (int j = 0; j < 32; ++j) still |= (uint32_t)(__uint_as_float(v[j]) < cut) << j;
-                                m &= still;
-                                if (__any_sync(0xffffffffu, __popc(m) > S::QD)) {
-                                    uint32_t mm = __reduce_or_sync(0xffffffffu, m);
-                                    while (mm != 0u) {
-                                        const int j = __ffs(mm) - 1;
-                                        mm &= mm - 1u;
-                                        const float d = __uint_as_float(tmem_ld1(taddr + ch * 32 + j));
-                                        int32_t xs = NET_EMPTY;
-                                        uint32_t xr = 0u;
-                                        if (((m >> j) & 1u) && d < cut) {
-                                            xs = (int32_t)(d + cq);
-                                            xr = (uint32_t)(rch + j);
-                                        }
-                                        net_insert(ls, lr, xs, xr);
-                                        set_cut();
-                                    }
-                                    share_cut();
-                                    continue;
+                            for (int g = 0; g < NG; ++g) left |= (uint32_t)(gm[g] < cut) << g;
+                            left = __reduce_or_sync(0xffffffffu, left);
+                            const float cm = cq + __uint_as_float(SCORE_MAGIC);
+#pragma unroll 1
+                            while (left != 0u) {
+                                const int col = (__ffs(left) - 1) * G;
+                                left &= left - 1u;
+                                if (__any_sync(0xffffffffu, queued > S::QD - G)) flush();
+                                uint32_t w[G], step[G];
+                                tmem_ld_group(taddr + ch * 32 + col, w);
+                                const int64_t r = rch + col;
+#pragma unroll
+                                for (int j = 0; j < G; ++j)
+                                    step[j] = queue_step(__uint_as_float(w[j]), cut);
+                                if (r + G > n_refs) {
+#pragma unroll
+                                    for (int j = 0; j < G; ++j)
+                                        if (r + j >= n_refs) step[j] = 0;
                                 }
-                            }
-                            const uint32_t mm = __reduce_or_sync(0xffffffffu, m);
-                            const uint32_t rel = (uint32_t)(rch - qbase);
+                                const uint32_t rel = (uint32_t)(r - qbase), at0 = smem_u32(queue);
+                                uint32_t at = at0 + (uint32_t)queued * (TC_BM * 4);
 #pragma unroll
-                            for (int g = 0; g < 32; g += 8) {
-                                if (((mm >> g) & 0xFFu) == 0u) continue;
-#pragma unroll
-                                for (int j = g; j < g + 8; ++j) {
-                                    if ((m >> j) & 1u) {
-                                        queue[queued * TC_BM] =
-                                            ((uint32_t)(int32_t)(__uint_as_float(v[j]) + cq) << TC_QBITS) | (rel + j);
-                                        ++queued;
-                                    }
+                                for (int j = 0; j < G; ++j) {
+                                    const uint32_t e = __float_as_uint(__uint_as_float(w[j]) + cm);
+                                    asm volatile("st.shared.u32 [%0], %1;" ::"r"(at), "r"((e << TC_QBITS) + (rel + j))
+                                                 : "memory");
+                                    at += step[j];
                                 }
+                                queued = (int)((at - at0) / (TC_BM * 4));
                             }
                         }
                         // every column of the tile is processed: the MMA may reuse the accumulator
