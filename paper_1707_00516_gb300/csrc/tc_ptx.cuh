@@ -205,14 +205,6 @@ __device__ __forceinline__ void tmem_fill16(uint32_t taddr, uint32_t v) {
         : "memory");
 }
 
-// 32 lanes x one 32-bit column (every lane its own row).
-__device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
-    uint32_t v;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    return v;
-}
-
 // 32 lanes x 2 or 4 consecutive columns.
 __device__ __forceinline__ void tmem_ld_group(uint32_t taddr, uint32_t (&v)[2]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(taddr));
