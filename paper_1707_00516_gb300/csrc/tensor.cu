@@ -25,7 +25,8 @@
 //   warp 0       TMA producer (one lane)
 //   warp 1       TMEM allocation + MMA issue (one lane)
 //   warps 2..5   epilogue: TMEM -> registers -> score filter -> per-query
-//                top-k (thread = query), hit list or full score matrix
+//                top-k (thread = query), hit list or full score matrix; a second
+//                set as the last four warps where ES = 2
 //   warps 6..    packed-reference launches only (PK): expansion of the packed
 //                reference stage into the FP8 stage (see expand_stage)
 // Two accumulators (2 x 256 TMEM columns) let the epilogue of one reference
@@ -44,7 +45,7 @@ namespace {
 
 constexpr int TC_BM = 128;          // queries per tile
 constexpr int TC_BK = 128;          // loci (bytes) per stage
-constexpr int TC_THREADS = 192;     // producer, MMA issuer, 4 epilogue warps
+constexpr int TC_THREADS = 192;     // producer, MMA issuer, 4 epilogue warps (a second set: 128 more)
 // PK: warps expanding packed references, after the 6 others.  Blocks of 257 to
 // 384 threads get at most 168 registers a thread, which the 16-slot top-k
 // fits (4 expanding warps) and the 32-slot one does not (2).
@@ -65,6 +66,21 @@ constexpr int SC_LD = 36;
 constexpr uint32_t SC_BYTES = 4 * 32 * SC_LD * 4;
 constexpr uint64_t RENDEZVOUS_NS = 50000000ull;  // 50 ms per panel entry, then go on alone
 
+// What a launch's epilogue does with the scores (its own instances: lists take
+// 32 to 64 registers a thread, transpose buffers a stage).
+enum { MODE_TOPK, MODE_SCORES, MODE_HITS };
+
+// Epilogue sets ES: for hit launches two sets of four warps, one an accumulator
+// (even and odd tiles): one set is one warp a scheduler, whose latencies
+// nothing hides (512 queries x 1M references, N = 1024, 0.6 hits a 32-column
+// chunk, a call: 212 -> 203 us).  One for top-k -- two sets' own lists take
+// twice the insertions, and their cuts come later (500 queries x 2M, N = 2048,
+// k = 16: 604 -> 658 us) -- and for full matrices, which gain nothing (500 x
+// 60,001 uint32: 55.9 and 56.1).
+__host__ __device__ constexpr int tc_threads(int km, bool pk, int es) {
+    return TC_THREADS + (pk ? pk_threads(km) : 0) + (es - 1) * 128;
+}
+
 // Kernel variants: references per tile (the MMA's N) and pipeline depth (as
 // many stages as shared memory holds: the pipeline is latency-bound, and on
 // GB300 going from 3 to 4 stages took the FP4 2048 x 20M launch from 27.5 to
@@ -77,17 +93,19 @@ constexpr uint64_t RENDEZVOUS_NS = 50000000ull;  // 50 ms per panel entry, then 
 //             stage, 7 stages (FP8 32 KB, FP4 30 KB a stage)
 //   SC (full-matrix launches): one stage less where the transpose buffers
 //   (SC_BYTES) would not fit beside the ring
-template <int BN, bool PK = false, bool CG2 = false, bool SC = false>
+template <int BN, bool PK = false, bool CG2 = false, int MODE = MODE_TOPK>
 struct TcShape {
+    static constexpr bool SC = MODE == MODE_SCORES;
     static constexpr int RING = CG2 ? 7 : BN == 128 ? 6 : (BN == 224 && !PK) ? 5 : 4;
     static constexpr int STAGES = RING - (SC && (BN == 224) != PK ? 1 : 0);
     static constexpr uint32_t B_BYTES = (uint32_t)(CG2 ? BN / 2 : BN) * TC_BK;
     static constexpr uint32_t TMEM_COLS = BN == 128 ? 256 : 512;
     // beside the ring: transpose buffers, or the candidate queues (QD entries
-    // a query row: what the fullest rings leave)
-    static constexpr int QD = CG2 && BN == 256 ? 3 : 11;
+    // a query row and epilogue set: what the fullest rings leave)
+    static constexpr int ES = MODE == MODE_HITS ? 2 : 1;
+    static constexpr int QD = ES == 2 ? (BN == 224 && !PK ? 5 : 8) : CG2 && BN == 256 ? 3 : 11;
     static constexpr int QG = QD < 8 ? 2 : 4;  // columns queued at a time, while QD - QG or fewer are
-    static constexpr uint32_t EX_BYTES = SC ? SC_BYTES : (uint32_t)QD * TC_BM * 4;
+    static constexpr uint32_t EX_BYTES = SC ? SC_BYTES : (uint32_t)(ES * QD) * TC_BM * 4;
 };
 
 // One database ("panel") of a launch, with its schedule (TcSched).
@@ -452,7 +470,7 @@ __device__ __forceinline__ GroupWork group_work(const TensorArgs &a, int64_t wg,
 // Hits take the same way to the queues as top-k candidates; appended chunk by
 // chunk, each waited for an atomic on the list's counter and ran code unrolled
 // over the columns (512 queries x 1M references, N = 1024, 0.6 hits a chunk:
-// HITS_BEFORE).
+// a call 226 -> 212 us).
 __device__ __forceinline__ void append_hits(const TensorArgs &args, const uint32_t *queue, int queued, int64_t qbase,
                                             int64_t q, int lane) {
     const uint32_t total = __reduce_add_sync(0xffffffffu, (uint32_t)queued);
@@ -595,13 +613,15 @@ __device__ __forceinline__ void expand_stage_f4(const uint8_t *sp, uint8_t *sb, 
 // which leaves room for 7 stages.  Both CTAs' loads complete on the even
 // CTA's full barrier; its commits release both CTAs' stages and accumulators;
 // both epilogues release an accumulator on the even CTA's barrier.
-// SC: full-matrix launches (EPI_SCORES*), with the transpose buffers of
-// store_scores; the others filter into top-k lists (EPI_TOPK) or hits.
-template <int BN, bool PAIR, int KM, bool PK, bool F4, bool CG2 = false, bool SC = false>
-__global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS, 1)
+// MODE: full-matrix launches (EPI_SCORES*) store through the transpose buffers
+// of store_scores; the others filter into top-k lists or hits.
+template <int BN, bool PAIR, int KM, bool PK, bool F4, bool CG2 = false, int MODE = MODE_TOPK>
+__global__ void __launch_bounds__(tc_threads(KM, PK, TcShape<BN, PK, CG2, MODE>::ES), 1)
     tensor_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TensorArgs args) {
-    using S = TcShape<BN, PK, CG2, SC>;
-    static_assert(!SC || (KM == 16 && !CG2 && BN != 128), "full-matrix launches: the single-call shapes");
+    using S = TcShape<BN, PK, CG2, MODE>;
+    constexpr bool SC = MODE == MODE_SCORES;
+    constexpr bool topk = MODE == MODE_TOPK;
+    static_assert(topk || (KM == 16 && !CG2 && BN != 128), "full-matrix and hit launches: the single-call shapes");
     static_assert(!CG2 || (PAIR && !PK), "2-SM MMA launches are paired, over an operand copy");
     static_assert(F4 ? BN == TC_BN4 : BN != TC_BN4, "FP4 launches use 224-reference tiles, FP8 ones 256 or 128");
     static_assert(!PAIR || BN != 128, "paired launches use 256- or 224-reference tiles");
@@ -845,7 +865,7 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                 tc_commit(smem_u32(&ctl->done));
             mbar_drain(smem_u32(&ctl->done), 0, args.status, 5);
         }
-    } else if (PK && warp >= 6) {
+    } else if (PK && warp >= 6 && warp < 6 + pk_threads(KM) / 32) {
         // ---------------- PK: reference expansion, warps 6.. ----------------
         const int t = tid - 192;
         int stage = 0;
@@ -880,18 +900,20 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
             }
         }
     } else {
-        // ---------------- epilogue: warps 2..5 ----------------
+        // ---------------- epilogue: warps 2..5 (and the last four) ----------------
+        constexpr int ES = S::ES;
+        const int set = warp < 6 ? 0 : 1;
         const int quad = warp & 3;            // TMEM lane quadrant this warp may access
         const int row = quad * 32 + lane;     // query row within the tile
         const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
         const float tplus1 = args.threshold == 0xFFFFFFFFu ? __int_as_float(0x7f800000) : (float)args.threshold + 1.0f;
         const int k = args.k;
-        const bool topk = !SC && args.epi == EPI_TOPK;
         // every row of the output starts on a 16-byte boundary
         const bool vec = SC && (reinterpret_cast<uintptr_t>(args.out) & 15) == 0 &&
                          ((args.ld_out * (args.epi == EPI_SCORES16 ? 2 : 4)) & 15) == 0;
-        int acc = 0;
+        int acc = set;
         uint32_t acc_phase = 0;
+        int64_t tiles = 0;  // of the walk so far
         int32_t ls[KM];   // this thread's top-k scores (see net_insert)
         uint32_t lr[KM];  // and their references
         bool ok = true;
@@ -957,7 +979,7 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                         }
                     };
                     set_cut();
-                    uint32_t *queue = reinterpret_cast<uint32_t *>(sT) + row;  // entry i at i * TC_BM (see queue_insert)
+                    uint32_t *queue = reinterpret_cast<uint32_t *>(sT) + set * S::QD * TC_BM + row;  // entry i at i * TC_BM (see queue_insert)
                     int queued = 0;
                     int64_t qbase = rc * BN;
                     auto flush = [&]() {
@@ -970,7 +992,7 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                         }
                         queued = 0;
                     };
-                    for (int64_t rt = rc; rt < re; ++rt) {
+                    for (int64_t rt = rc + (ES == 2 ? (tiles & 1) ^ set : 0); rt < re; rt += ES) {
                         const bool got = mbar_wait(smem_u32(&ctl->tfull[acc]), acc_phase, abort_flag, args.status, 6);
                         __syncwarp();
                         if (!__all_sync(0xffffffffu, got)) {
@@ -1069,11 +1091,14 @@ __global__ void __launch_bounds__(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS,
                             mbar_arrive_cluster(mapa_rank(smem_u32(&ctl->tempty[acc]), 0));
                         else
                             mbar_arrive(smem_u32(&ctl->tempty[acc]));
-                        if (++acc == 2) {
+                        if (ES == 2) {
+                            acc_phase ^= 1u;
+                        } else if (++acc == 2) {
                             acc = 0;
                             acc_phase ^= 1u;
                         }
                     }
+                    tiles += re - rc;
                     if (!SC && ok) {
                         flush();
                         if (topk) list_save(slot, ls, lr, k);
@@ -1307,9 +1332,9 @@ __global__ void prep_jobs_kernel(const PrepJob *__restrict__ jobs, int64_t n_job
     }
 }
 
-template <int BN, bool PK = false, bool CG2 = false, bool SC = false>
+template <int BN, bool PK = false, bool CG2 = false, int MODE = MODE_TOPK>
 size_t tensor_smem(bool f4 = false) {
-    using S = TcShape<BN, PK, CG2, SC>;
+    using S = TcShape<BN, PK, CG2, MODE>;
     return 1024 + S::STAGES * (size_t)(TC_A_BYTES + S::B_BYTES + (PK ? pk_stage_bytes(BN, f4) : 0)) +
            S::EX_BYTES + 256;
 }
@@ -1459,18 +1484,18 @@ int tensor_grid_target(int device) {
 
 namespace {
 
-// One launch of tensor_kernel<BN, PAIR, KM, PK, F4, CG2, SC> over n_groups work
+// One launch of tensor_kernel<BN, PAIR, KM, PK, F4, CG2, MODE> over n_groups work
 // groups (2-CTA clusters when paired).
-template <int BN, bool PAIR, int KM, bool PK = false, bool F4 = false, bool CG2 = false, bool SC = false>
-cudaError_t launch_variant(const TcMaps &maps, const TensorArgs &a, int32_t n_groups, int epi, cudaStream_t s) {
-    const size_t smem = tensor_smem<BN, PK, CG2, SC>(F4);
-    cudaError_t e = cudaFuncSetAttribute(tensor_kernel<BN, PAIR, KM, PK, F4, CG2, SC>,
+template <int BN, bool PAIR, int KM, bool PK = false, bool F4 = false, bool CG2 = false, int MODE = MODE_TOPK>
+cudaError_t launch_variant(const TcMaps &maps, const TensorArgs &a, int32_t n_groups, cudaStream_t s) {
+    const size_t smem = tensor_smem<BN, PK, CG2, MODE>(F4);
+    cudaError_t e = cudaFuncSetAttribute(tensor_kernel<BN, PAIR, KM, PK, F4, CG2, MODE>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3((PAIR ? 2 : 1) * n_groups);
-    cfg.blockDim = dim3(PK ? TC_THREADS + pk_threads(KM) : TC_THREADS);
+    cfg.blockDim = dim3(tc_threads(KM, PK, TcShape<BN, PK, CG2, MODE>::ES));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -1480,7 +1505,19 @@ cudaError_t launch_variant(const TcMaps &maps, const TensorArgs &a, int32_t n_gr
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = PAIR ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, tensor_kernel<BN, PAIR, KM, PK, F4, CG2, SC>, maps, a);
+    return cudaLaunchKernelEx(&cfg, tensor_kernel<BN, PAIR, KM, PK, F4, CG2, MODE>, maps, a);
+}
+
+// Full-matrix and hit launches: the shapes of single calls.
+template <int MODE>
+cudaError_t launch_single(const TcMaps &maps, const TensorArgs &a, const TcLaunch &L, cudaStream_t s) {
+    if (L.f4)
+        return L.pk     ? launch_variant<TC_BN4, false, 16, true, true, false, MODE>(maps, a, L.n_groups, s)
+               : L.pair ? launch_variant<TC_BN4, true, 16, false, true, false, MODE>(maps, a, L.n_groups, s)
+                        : launch_variant<TC_BN4, false, 16, false, true, false, MODE>(maps, a, L.n_groups, s);
+    return L.pk     ? launch_variant<256, false, 16, true, false, false, MODE>(maps, a, L.n_groups, s)
+           : L.pair ? launch_variant<256, true, 16, false, false, false, MODE>(maps, a, L.n_groups, s)
+                    : launch_variant<256, false, 16, false, false, false, MODE>(maps, a, L.n_groups, s);
 }
 
 }  // namespace
@@ -1523,47 +1560,41 @@ cudaError_t launch_tensor_multi(int bn, const TcLaunch &L, cudaStream_t s) {
     a.partial = L.partial;
     a.status = L.status;
     a.arrive = L.arrive;
-    if (L.epi == EPI_SCORES16 || L.epi == EPI_SCORES32) {
+    if (L.epi != EPI_TOPK) {
         if (L.cg2 || (L.pk && L.pair) || (!L.f4 && bn != 256)) return cudaErrorInvalidValue;
-        if (L.f4)
-            return L.pk     ? launch_variant<TC_BN4, false, 16, true, true, false, true>(maps, a, L.n_groups, L.epi, s)
-                   : L.pair ? launch_variant<TC_BN4, true, 16, false, true, false, true>(maps, a, L.n_groups, L.epi, s)
-                            : launch_variant<TC_BN4, false, 16, false, true, false, true>(maps, a, L.n_groups, L.epi, s);
-        return L.pk     ? launch_variant<256, false, 16, true, false, false, true>(maps, a, L.n_groups, L.epi, s)
-               : L.pair ? launch_variant<256, true, 16, false, false, false, true>(maps, a, L.n_groups, L.epi, s)
-                        : launch_variant<256, false, 16, false, false, false, true>(maps, a, L.n_groups, L.epi, s);
+        return L.epi == EPI_HITS ? launch_single<MODE_HITS>(maps, a, L, s) : launch_single<MODE_SCORES>(maps, a, L, s);
     }
     // 16-slot lists when k allows (half the insert network, 32 fewer registers)
-    const bool k16 = L.epi != EPI_TOPK || L.k <= 16;
+    const bool k16 = L.k <= 16;
     if (L.f4) {  // 224-reference tiles whatever bn says
         if (L.pk) {
             if (L.pair) return cudaErrorInvalidValue;
-            return k16 ? launch_variant<TC_BN4, false, 16, true, true>(maps, a, L.n_groups, L.epi, s)
-                       : launch_variant<TC_BN4, false, 32, true, true>(maps, a, L.n_groups, L.epi, s);
+            return k16 ? launch_variant<TC_BN4, false, 16, true, true>(maps, a, L.n_groups, s)
+                       : launch_variant<TC_BN4, false, 32, true, true>(maps, a, L.n_groups, s);
         }
         if (L.pair && L.cg2)
-            return k16 ? launch_variant<TC_BN4, true, 16, false, true, true>(maps, a, L.n_groups, L.epi, s)
-                       : launch_variant<TC_BN4, true, 32, false, true, true>(maps, a, L.n_groups, L.epi, s);
-        if (L.pair) return k16 ? launch_variant<TC_BN4, true, 16, false, true>(maps, a, L.n_groups, L.epi, s)
-                               : launch_variant<TC_BN4, true, 32, false, true>(maps, a, L.n_groups, L.epi, s);
-        return k16 ? launch_variant<TC_BN4, false, 16, false, true>(maps, a, L.n_groups, L.epi, s)
-                   : launch_variant<TC_BN4, false, 32, false, true>(maps, a, L.n_groups, L.epi, s);
+            return k16 ? launch_variant<TC_BN4, true, 16, false, true, true>(maps, a, L.n_groups, s)
+                       : launch_variant<TC_BN4, true, 32, false, true, true>(maps, a, L.n_groups, s);
+        if (L.pair) return k16 ? launch_variant<TC_BN4, true, 16, false, true>(maps, a, L.n_groups, s)
+                               : launch_variant<TC_BN4, true, 32, false, true>(maps, a, L.n_groups, s);
+        return k16 ? launch_variant<TC_BN4, false, 16, false, true>(maps, a, L.n_groups, s)
+                   : launch_variant<TC_BN4, false, 32, false, true>(maps, a, L.n_groups, s);
     }
     if (L.pair && bn != 256) return cudaErrorInvalidValue;
     if (L.pk) {
         if (L.pair || bn != 256) return cudaErrorInvalidValue;
-        return k16 ? launch_variant<256, false, 16, true>(maps, a, L.n_groups, L.epi, s)
-                   : launch_variant<256, false, 32, true>(maps, a, L.n_groups, L.epi, s);
+        return k16 ? launch_variant<256, false, 16, true>(maps, a, L.n_groups, s)
+                   : launch_variant<256, false, 32, true>(maps, a, L.n_groups, s);
     }
     if (L.pair && L.cg2)
-        return k16 ? launch_variant<256, true, 16, false, false, true>(maps, a, L.n_groups, L.epi, s)
-                   : launch_variant<256, true, 32, false, false, true>(maps, a, L.n_groups, L.epi, s);
-    if (L.pair) return k16 ? launch_variant<256, true, 16>(maps, a, L.n_groups, L.epi, s)
-                           : launch_variant<256, true, 32>(maps, a, L.n_groups, L.epi, s);
-    if (bn == 128) return k16 ? launch_variant<128, false, 16>(maps, a, L.n_groups, L.epi, s)
-                              : launch_variant<128, false, 32>(maps, a, L.n_groups, L.epi, s);
-    return k16 ? launch_variant<256, false, 16>(maps, a, L.n_groups, L.epi, s)
-               : launch_variant<256, false, 32>(maps, a, L.n_groups, L.epi, s);
+        return k16 ? launch_variant<256, true, 16, false, false, true>(maps, a, L.n_groups, s)
+                   : launch_variant<256, true, 32, false, false, true>(maps, a, L.n_groups, s);
+    if (L.pair) return k16 ? launch_variant<256, true, 16>(maps, a, L.n_groups, s)
+                           : launch_variant<256, true, 32>(maps, a, L.n_groups, s);
+    if (bn == 128) return k16 ? launch_variant<128, false, 16>(maps, a, L.n_groups, s)
+                              : launch_variant<128, false, 32>(maps, a, L.n_groups, s);
+    return k16 ? launch_variant<256, false, 16>(maps, a, L.n_groups, s)
+               : launch_variant<256, false, 32>(maps, a, L.n_groups, s);
 }
 
 }  // namespace fastid
