@@ -648,7 +648,6 @@ fastid_status topk_few(fastid_ctx *ctx, const fastid_refdb *db, const FewShape &
     L.k = k;
     L.n_slots = slices;
     L.status = ctx->dev_status;
-    L.dependent = 1;
     L.sched[0].n_qq = 1;
     L.sched[0].a = 1;
     L.sched[0].b = slices;

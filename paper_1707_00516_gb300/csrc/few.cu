@@ -277,8 +277,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
         for (int c = 0; c < (int)FQ_A_COL; c += 16) tmem_fill16(lanes + c, 0u);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
-    // (everything up to here ran beside the seed kernel)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();  // (everything up to here ran beside the seed kernel)
     const float INF = __int_as_float(0x7f800000);
     const float t1 = A.threshold == 0xFFFFFFFFu ? INF : (float)A.threshold + 1.0f;
     if (tid < FQ_N) {
@@ -617,7 +616,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
         }
     }
 
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the merge, which waits for these results
+    pdl_trigger();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -638,7 +637,7 @@ __global__ void __launch_bounds__(FQ_SEED_WARPS * 32)
                     const uint8_t *__restrict__ modes, int32_t kbytes, uint8_t *__restrict__ out,
                     float *__restrict__ qconst, const SharedCut cut, const uint64_t *__restrict__ refs, int64_t stride,
                     int sample, int k, int32_t *__restrict__ pub, int32_t slices) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the compare kernel waits for this one's results)
+    pdl_trigger();
     __shared__ uint32_t sc[FQ_SAMPLE_MAX];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t r = blockIdx.x;

@@ -151,6 +151,7 @@ __global__ void query_prep_kernel(const uint64_t *__restrict__ q, int64_t ld_q, 
                                   int32_t n_words, const uint8_t *__restrict__ modes,
                                   uint32_t *__restrict__ q32, int64_t n_q_pad, int64_t ld32,
                                   QueryCoef *__restrict__ coef) {
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int64_t ld64 = ld32 / 2;

@@ -128,6 +128,7 @@ __device__ __forceinline__ uint4 lds128_once(const uint32_t *p) {
 
 template <int EPI, int JQ>
 __global__ void __launch_bounds__(PL_THREADS, JQ > 2 ? 2 : 3) plain_kernel(const PlainArgs args) {
+    pdl_wait();
     constexpr int TQ = 16 * JQ;
     constexpr int JC = JQ < 4 ? JQ : 4;  // query columns a step
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -479,8 +480,7 @@ cudaError_t launch_plain(int epi, const uint32_t *refs32, const uint32_t *ref_no
     cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    fn<<<part.grid, PL_THREADS, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(fn, dim3((unsigned)part.grid), dim3(PL_THREADS), smem, s, a);
 }
 
 }  // namespace fastid

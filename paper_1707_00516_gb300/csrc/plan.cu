@@ -289,12 +289,12 @@ fastid_status fastid_plan_run(fastid_plan *plan, fastid_stream stream) {
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return pcuda(ctx, e, "cudaSetDevice");
     if (plan->n_queries == 0) return FASTID_OK;
-    e = launch_prep_jobs(plan->prep, plan->n_jobs_prep, s);
-    if (e != cudaSuccess) return pcuda(ctx, e, "batched operand preparation");
     if (plan->launch.arrive) {
         e = cudaMemsetAsync(plan->launch.arrive, 0, TC_MAXP * sizeof(unsigned int), s);
         if (e != cudaSuccess) return pcuda(ctx, e, "panel counters");
     }
+    e = launch_prep_jobs(plan->prep, plan->n_jobs_prep, s);
+    if (e != cudaSuccess) return pcuda(ctx, e, "batched operand preparation");
     e = launch_tensor_multi(plan->bn, plan->launch, s);
     if (e != cudaSuccess) return pcuda(ctx, e, "batched compare launch");
     e = launch_merge_sched(plan->partial, plan->launch, plan->merge, plan->n_jobs_merge, nullptr, nullptr, s);

@@ -56,6 +56,7 @@ __device__ int64_t cta_of(const Partition &P, int64_t u) {
 __global__ void topk_merge_kernel(const uint64_t *__restrict__ partial, Partition P, int64_t n_q, int32_t k, int W,
                                   uint32_t *__restrict__ out_scores, int64_t *__restrict__ out_idx) {
     __shared__ uint64_t sm[MERGE_MAX_WARPS][32];
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int64_t q = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) / W;
@@ -118,7 +119,7 @@ __global__ void topk_merge_sched_kernel(const uint64_t *__restrict__ partial, co
                                         const MergeJob *__restrict__ jobs, int64_t n_jobs, int W,
                                         uint32_t *__restrict__ out_s, int64_t *__restrict__ out_i) {
     __shared__ uint64_t sm[MERGE_MAX_WARPS][32];
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // (returns at once in an ordinary launch)
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int64_t j = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) / W;
@@ -257,6 +258,8 @@ __global__ void __launch_bounds__(RS_THREADS) hits_count_kernel(const unsigned l
                                                                 const int64_t *__restrict__ hq,
                                                                 const int64_t *__restrict__ hr, int r_bits,
                                                                 uint32_t *__restrict__ table) {
+    pdl_trigger();
+    pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned long long c = *count;
         *count_out = (int64_t)c;
@@ -288,6 +291,8 @@ __global__ void __launch_bounds__(RS_THREADS)
                         const uint64_t *__restrict__ src_k, const int64_t *__restrict__ src_r,
                         const uint32_t *__restrict__ src_v, uint64_t *__restrict__ dst_k, int64_t *__restrict__ dst_r,
                         uint32_t *__restrict__ dst_v) {
+    pdl_trigger();
+    pdl_wait();
     const int64_t n = hits_live(count, capacity);
     const int sh = rs_shift(n);
     const int64_t b0 = (int64_t)blockIdx.x << sh, b1 = min(n, b0 + ((int64_t)1 << sh));
@@ -436,9 +441,8 @@ cudaError_t launch_topk_merge(const uint64_t *partial, const Partition &part, in
     if (n_q == 0) return cudaSuccess;
     const int64_t n_qt = part.n_qt;
     const int W = merge_warps(n_q, (part.grid + n_qt - 1) / n_qt + 1), per = merge_block_warps(W) / W;
-    topk_merge_kernel<<<(unsigned)((n_q + per - 1) / per), per * W * 32, 0, s>>>(partial, part, n_q, k, W, out_scores,
-                                                                                out_idx);
-    return cudaGetLastError();
+    return launch_dependent(topk_merge_kernel, dim3((unsigned)((n_q + per - 1) / per)), dim3(per * W * 32), 0, s, partial,
+                            part, n_q, k, W, out_scores, out_idx);
 }
 
 cudaError_t launch_merge_sched(const uint64_t *partial, const TcLaunch &L, const MergeJob *jobs, int64_t n_jobs,
@@ -460,11 +464,7 @@ cudaError_t launch_merge_sched(const uint64_t *partial, const TcLaunch &L, const
         n_lists = std::max<int64_t>(n_lists, L.sched[p].b + (L.sched[p].t_groups > 0 ? 1 : 0));
     const int W = merge_warps(n_jobs, n_lists), per = merge_block_warps(W) / W;
     const dim3 grid((unsigned)((n_jobs + per - 1) / per)), block(per * W * 32);
-    if (L.dependent)
-        return launch_dependent(topk_merge_sched_kernel, grid, block, 0, s, partial, M, jobs, n_jobs, W, out_scores,
-                                out_idx);
-    topk_merge_sched_kernel<<<grid, block, 0, s>>>(partial, M, jobs, n_jobs, W, out_scores, out_idx);
-    return cudaGetLastError();
+    return launch_dependent(topk_merge_sched_kernel, grid, block, 0, s, partial, M, jobs, n_jobs, W, out_scores, out_idx);
 }
 
 cudaError_t launch_topk_fold(uint32_t *run_s, int64_t *run_i, const uint32_t *blk_s, const int64_t *blk_i,
@@ -495,27 +495,30 @@ cudaError_t launch_hits_finish(void *aux, int64_t capacity, int64_t n_q, int64_t
     uint64_t *tk = reinterpret_cast<uint64_t *>(base + L.keys);
     uint32_t *tv = reinterpret_cast<uint32_t *>(base + L.vals);
     const unsigned grid = (unsigned)std::max<int64_t>(1, nb);
-    hits_count_kernel<<<grid, RS_THREADS, 0, s>>>(count, capacity, count_out, status, hit_q, hit_r, r_bits, table);
-    if (capacity == 0) return cudaGetLastError();
+    const dim3 blocks(grid), threads(RS_THREADS);
+    cudaError_t e = launch_dependent(hits_count_kernel, blocks, threads, 0, s, count, capacity, count_out, status, hit_q,
+                                     hit_r, r_bits, table);
+    if (capacity == 0) return e;
     uint64_t *hk = reinterpret_cast<uint64_t *>(hit_q);
-    for (int p = 0; p < passes; ++p) {
+    for (int p = 0; p < passes && e == cudaSuccess; ++p) {
         const uint32_t *now = table + (int64_t)p * nb * RS_DIGITS;
-        uint32_t *next = table + (int64_t)(p + 1) * nb * RS_DIGITS;
+        uint32_t *next = p + 1 < passes ? table + (int64_t)(p + 1) * nb * RS_DIGITS : nullptr;
         const int shift = p * RS_BITS;
+        int64_t *none = nullptr;
         if (p == 0)
-            hits_scatter_kernel<true, false><<<grid, RS_THREADS, 0, s>>>(count, capacity, r_bits, shift, now, next, hk,
-                                                                         hit_r, hit_score, tk, nullptr, tv);
+            e = launch_dependent(hits_scatter_kernel<true, false>, blocks, threads, 0, s, count, capacity, r_bits, shift,
+                                 now, next, hk, hit_r, hit_score, tk, none, tv);
         else if (p + 1 == passes)
-            hits_scatter_kernel<false, true><<<grid, RS_THREADS, 0, s>>>(count, capacity, r_bits, shift, now, nullptr,
-                                                                         tk, nullptr, tv, hk, hit_r, hit_score);
+            e = launch_dependent(hits_scatter_kernel<false, true>, blocks, threads, 0, s, count, capacity, r_bits, shift,
+                                 now, next, tk, none, tv, hk, hit_r, hit_score);
         else if (p & 1)
-            hits_scatter_kernel<false, false><<<grid, RS_THREADS, 0, s>>>(count, capacity, r_bits, shift, now, next,
-                                                                          tk, nullptr, tv, hk, nullptr, hit_score);
+            e = launch_dependent(hits_scatter_kernel<false, false>, blocks, threads, 0, s, count, capacity, r_bits,
+                                 shift, now, next, tk, none, tv, hk, none, hit_score);
         else
-            hits_scatter_kernel<false, false><<<grid, RS_THREADS, 0, s>>>(count, capacity, r_bits, shift, now, next,
-                                                                          hk, nullptr, hit_score, tk, nullptr, tv);
+            e = launch_dependent(hits_scatter_kernel<false, false>, blocks, threads, 0, s, count, capacity, r_bits,
+                                 shift, now, next, hk, none, hit_score, tk, none, tv);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace fastid

@@ -696,6 +696,8 @@ __global__ void __launch_bounds__(tc_threads(KM, PK, TcShape<BN, PK, CG2, MODE>:
         tc_fence_after();
     }
 
+    pdl_wait();  // (everything up to here ran beside the query preparation)
+
     if (warp == 0) {
         // ---------------- TMA producer ----------------
         // Per stage: one wait for the slot (inline when it is already free),
@@ -1108,6 +1110,7 @@ __global__ void __launch_bounds__(tc_threads(KM, PK, TcShape<BN, PK, CG2, MODE>:
         }
     }
 
+    pdl_trigger();
     tc_fence_before();
     __syncthreads();
     if (PAIR) cluster_sync();  // neither CTA leaves while the other may still address it
@@ -1288,6 +1291,7 @@ __global__ void queries_e2m1_kernel(const uint64_t *__restrict__ q, int64_t ld_q
                                     int32_t n_loci, const uint8_t *__restrict__ modes, int64_t n_q_pad,
                                     int32_t kbytes, uint8_t *__restrict__ out, float *__restrict__ qconst,
                                     int64_t spread, const SharedCut cut) {
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n_q_pad; r += warps_total) {
@@ -1304,6 +1308,7 @@ __global__ void queries_e4m3_kernel(const uint64_t *__restrict__ q, int64_t ld_q
                                     int32_t n_loci, const uint8_t *__restrict__ modes, int64_t n_q_pad,
                                     int32_t kpad, uint8_t *__restrict__ out, float *__restrict__ qconst,
                                     uint32_t one, bool pk, int64_t spread, const SharedCut cut) {
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n_q_pad; r += warps_total) {
@@ -1318,6 +1323,7 @@ __global__ void queries_e4m3_kernel(const uint64_t *__restrict__ q, int64_t ld_q
 
 // Batched form: one job per operand row of every panel.
 __global__ void prep_jobs_kernel(const PrepJob *__restrict__ jobs, int64_t n_jobs) {
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t j = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < n_jobs; j += warps_total) {
@@ -1498,13 +1504,15 @@ cudaError_t launch_variant(const TcMaps &maps, const TensorArgs &a, int32_t n_gr
     cfg.blockDim = dim3(tc_threads(KM, PK, TcShape<BN, PK, CG2, MODE>::ES));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = PAIR ? 2 : 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // after the query preparation (see launch_dependent)
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = PAIR ? 2 : 1;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = PAIR ? 1 : 0;
+    cfg.numAttrs = PAIR ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, tensor_kernel<BN, PAIR, KM, PK, F4, CG2, MODE>, maps, a);
 }
 
