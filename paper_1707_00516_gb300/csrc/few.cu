@@ -52,8 +52,8 @@
 // merging warps), so that few candidates ever arrive.
 //
 // Measured (fastid_topk, 20M references, N = 2048, us; the tensor kernel over
-// packed rows before -> this form): 1 query 1930 -> 1080, 48 mixtures 2000 ->
-// 1200, 64 at k = 32 2400 -> 1540.  HBM is the floor at 754; the SM's issue
+// packed rows before -> this form): 1 query 1930 -> 1043, 48 mixtures 2000 ->
+// 1149, 64 at k = 32 2400 -> 1404.  HBM is the floor at 754; the SM's issue
 // slots set the pace (expansion ~2000 of ~3900 warp instructions a tile).
 #include <algorithm>
 #include <cstring>
@@ -571,32 +571,46 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
                 // any d < cut: the sign of d - cut (an infinite cut keeps its
                 // sign, and D holds no NaN), ORed
                 const float4 *c4 = reinterpret_cast<const float4 *>(cut + cb);
-                uint32_t sign = 0;
+                uint32_t d[32], any = 0;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const float4 c = c4[j];
-                    sign |= __float_as_uint(__uint_as_float(v[4 * j]) - c.x) | __float_as_uint(__uint_as_float(v[4 * j + 1]) - c.y);
-                    sign |= __float_as_uint(__uint_as_float(v[4 * j + 2]) - c.z) | __float_as_uint(__uint_as_float(v[4 * j + 3]) - c.w);
+                    d[4 * j] = __float_as_uint(__uint_as_float(v[4 * j]) - c.x);
+                    d[4 * j + 1] = __float_as_uint(__uint_as_float(v[4 * j + 1]) - c.y);
+                    d[4 * j + 2] = __float_as_uint(__uint_as_float(v[4 * j + 2]) - c.z);
+                    d[4 * j + 3] = __float_as_uint(__uint_as_float(v[4 * j + 3]) - c.w);
+                    any |= d[4 * j] | d[4 * j + 1];
+                    any |= d[4 * j + 2] | d[4 * j + 3];
                 }
-                if (!__any_sync(0xffffffffu, live && (int32_t)sign < 0)) continue;
+                if (!__any_sync(0xffffffffu, live && (int32_t)any < 0)) continue;
+                // A short loop over the groups of four columns that some lane
+                // needs, re-read from TMEM: unrolled over the 32 columns, the code was
+                // fetched anew each time (2048 loci, 48 queries, k = 32: 3M
+                // references 353 -> 301 us, 20M 1273 -> 1206).
                 uint32_t m = 0;
 #pragma unroll
-                for (int j = 0; j < 32; ++j) m |= (uint32_t)(__uint_as_float(v[j]) < cut[cb + j]) << j;
-                if (!live) m = 0;
-                const uint32_t mm = __reduce_or_sync(0xffffffffu, m);
+                for (int j = 0; j < 8; ++j)
+                    m |= ((d[4 * j] | d[4 * j + 1] | d[4 * j + 2] | d[4 * j + 3]) >> 31) << j;
+                m = __reduce_or_sync(0xffffffffu, live ? m : 0u);
+#pragma unroll 1
+                while (m != 0u) {
+                    const int q0 = cb + 4 * (__ffs(m) - 1);
+                    m &= m - 1u;
+                    uint32_t w[4];
+                    tmem_ld_group(taddr + q0, w);
+                    const float4 c = *reinterpret_cast<const float4 *>(cut + q0);
+                    const float cq[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
-                for (int g = 0; g < 32; g += 8) {
-                    if (((mm >> g) & 0xFFu) == 0u) continue;
-#pragma unroll
-                    for (int j = g; j < g + 8; ++j) {
-                        if ((m >> j) & 1u) {
-                            const int q = cb + j;
-                            const uint64_t key =
-                                make_key((uint32_t)(int32_t)(__uint_as_float(v[j]) + qc[q]), (uint32_t)r);
+                    for (int j = 0; j < 4; ++j) {
+                        const float x = __uint_as_float(w[j]);
+                        if (live && x < cq[j]) {
+                            const int q = q0 + j;
+                            const uint64_t key = make_key((uint32_t)(int32_t)(x + qc[q]), (uint32_t)r);
                             const uint32_t at = atomicAdd(&head[q], 1u);
                             ring_put(ring + q * FQ_QUEUE, tail + q, at, key, abort_flag, A.status);
                         }
                     }
+                    __syncwarp();
                 }
                 __syncwarp();
             }
