@@ -89,6 +89,11 @@ __host__ __device__ inline bool op_f4(int op) { return op == OP_FP4 || op == OP_
 //   2048         24.1/24.6   29.7/40.8    40.6/40.6   50.3/65.2
 // so the FP4 packed rows are never slower than an FP8 operand, and the FP4
 // copy wins from two query tiles on.
+// (Before the few-query form, few.cu, which takes up to 64 queries over the
+// packed rows in 1.04 to 1.40, and the cuts shared by a launch's slices.  One
+// query tile over a short database is even: 96 queries, k = 10 / 32, 500,000
+// references 111 / 147 us over the copy and 100 / 145 packed, 100,000 54 / 85
+// and 54 / 86.)
 constexpr int64_t AUTO_FP4_PACKED_MAX_Q = 128;
 int pick_operand(int form, bool has_fp8, bool has_fp4, int64_t n_q, bool slots16 = true);
 
