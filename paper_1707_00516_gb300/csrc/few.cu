@@ -132,7 +132,10 @@ static_assert(sizeof(FewSmem) <= 512, "control block");
 // cycles and the pipe holds one or two, so what the issuing warp does between
 // stages must not wait: the next stage's barrier and the next accumulator's
 // are tested first in the block and the answers (ready, room) read last, when
-// they have long arrived.
+// they have long arrived.  The answers are each lane's own: the warp votes on
+// them before it branches, as it does on everything that other warps or CTAs
+// change, because the two sides of such a branch meet at whole-warp
+// instructions (elect.sync, votes, reductions).
 template <bool FULL>
 __device__ __forceinline__ void mma_few(uint32_t d, uint32_t a, uint64_t b, uint64_t b2, uint32_t idesc, uint32_t sfa,
                                         uint32_t sfb, uint32_t acc, uint32_t commit, uint32_t next, uint32_t next_par,
@@ -341,7 +344,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
         uint32_t ready = 0, room = 1;
         bool ok = warp_wait(smem_u32(&ctl->bfull), 0, abort_flag, A.status, 23);
         for (uint32_t tt = first; tt < n_tiles && ok; tt += 2) {
-            if (!room) {
+            if (!__all_sync(0xffffffffu, room)) {
                 ok = warp_wait(smem_u32(&ctl->tempty[acc]), acc_phase ^ 1u, abort_flag, A.status, 24);
                 if (!ok) break;
             }
@@ -353,7 +356,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
             const uint32_t rb = smem_u32(&ctl->tempty[acc]);
             uint64_t b = bd0;
             for (uint32_t st = 0; st < n_st; ++st) {
-                if (!ready) {
+                if (!__all_sync(0xffffffffu, ready)) {
                     ok = warp_wait(af0 + 8 * as, aphase, abort_flag, A.status, 25);
                     if (!ok) break;
                 }
@@ -388,7 +391,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
         const int first_q = (int)y % A.n_q;
         int union_q = first_q;  // the query whose cut this slice bounds over all slices next
         for (bool last = false;;) {
-            const bool ended = *reinterpret_cast<volatile int *>(&ctl->finished) == 8;
+            const bool ended = __all_sync(0xffffffffu, *reinterpret_cast<volatile int *>(&ctl->finished) == 8);
             __threadfence_block();  // entries put in before the warps were through are seen below
             int64_t at = t_hi;  // every reference below tile `at` has been filtered
             for (int w = 0; w < 8; ++w) at = min(at, *reinterpret_cast<volatile int64_t *>(&ctl->tile[w]));
@@ -446,7 +449,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
                 if (kth != NET_EMPTY) c = fminf(c, (float)(strict ? kth : kth + 1));
                 *reinterpret_cast<volatile float *>(cut + mine) = c - qc[mine];
             }
-            if (last || *abort_flag) break;
+            if (__any_sync(0xffffffffu, last || *abort_flag != 0)) break;
             last = ended && !busy && least == 1u;  // one more look after the last entries
             least = busy && !ended ? FQ_MERGE_MIN : 1u;
             if (busy || ended) continue;
@@ -462,7 +465,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
                 for (int i = 0; i < FQ_SLICES_MAX / 32; ++i)
                     v[i] = 32 * i + lane < A.slices ? load_cut(A.pub + (int64_t)union_q * A.slices + 32 * i + lane)
                                                     : NET_EMPTY;
-                const int32_t now = load_cut(A.gcut + union_q);
+                const int32_t now = __shfl_sync(0xffffffffu, load_cut(A.gcut + union_q), 0);
                 int32_t lo = 0, hi = now == NET_EMPTY ? FASTID_MAX_LOCI : now;
                 auto at_most = [&](int32_t m) {
                     int n = 0;
@@ -552,6 +555,7 @@ __global__ void __launch_bounds__(FQ_THREADS, 1)
                 aphase ^= 1u;
             }
         }
+        __syncwarp();
         announce();
     } else {
         // ---------------- epilogue ----------------
