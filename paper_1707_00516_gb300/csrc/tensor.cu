@@ -993,6 +993,7 @@ __global__ void __launch_bounds__(tc_threads(KM, PK, TcShape<BN, PK, CG2, MODE>:
                             append_hits(args, queue, queued, qbase, q, lane);
                         }
                         queued = 0;
+                        __syncwarp();  // lanes took their own ways; what follows may be a whole-warp TMEM load
                     };
                     for (int64_t rt = rc + (ES == 2 ? (tiles & 1) ^ set : 0); rt < re; rt += ES) {
                         const bool got = mbar_wait(smem_u32(&ctl->tfull[acc]), acc_phase, abort_flag, args.status, 6);
