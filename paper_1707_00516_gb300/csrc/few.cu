@@ -208,13 +208,6 @@ __device__ __noinline__ void ring_put(uint64_t *ring, uint32_t *tail, uint32_t a
     *reinterpret_cast<volatile uint64_t *>(ring + (at & (FQ_QUEUE - 1))) = key;
 }
 
-// Whole-warp wait: every lane agrees on the outcome.
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint32_t *status,
-                                          uint32_t site) {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, site));
-}
-
 __global__ void __launch_bounds__(FQ_THREADS, 1)
     few_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_r, const FewArgs A) {
     extern __shared__ uint8_t smem_raw[];

@@ -789,6 +789,9 @@ __global__ void __launch_bounds__(tc_threads(KM, PK, TcShape<BN, PK, CG2, MODE>:
     } else if (warp == 1) {
         // ---------------- MMA issuer (2-SM pairs: the even CTA's) ----------------
         // The whole warp, converged; one elected lane issues (see tc_commit).
+        // The lanes vote on every wait (warp_wait): where one ran out, all of
+        // them leave together, and none is left at an elect.sync that the
+        // others never reach.
         // Per stage: one barrier wait (inline when the stage is already full),
         // the stage's descriptors as constant offsets from the first stage's,
         // four MMAs in one asm block, one commit (see mma_stage4).
@@ -815,20 +818,16 @@ __global__ void __launch_bounds__(tc_threads(KM, PK, TcShape<BN, PK, CG2, MODE>:
                     for (int32_t qq = W.q_lo; qq < W.q_hi && ok; ++qq) {
                         for (int64_t rt = rc; rt < re && ok; ++rt) {
                             const uint32_t tempty = smem_u32(&ctl->tempty[acc]);
-                            if (!mbar_try_wait(tempty, acc_phase ^ 1u)) {
-                                ok = mbar_wait(tempty, acc_phase ^ 1u, abort_flag, args.status, 3);
-                                if (!ok) break;
-                            }
+                            ok = warp_wait(tempty, acc_phase ^ 1u, abort_flag, args.status, 3);
+                            if (!ok) break;
                             tc_fence_after();  // the epilogue's reads of this accumulator come first
                             const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
                             for (int kb = 0; kb < n_kb; ++kb) {
                                 const uint32_t fb = full0 + 8u * stage;
-                                if (!mbar_try_wait(fb, phase)) {
-                                    ok = mbar_wait(fb, phase, abort_flag, args.status, 4);
-                                    if (!ok) break;
-                                }
-                                if (PK && !mbar_try_wait(bfull0 + 8u * stage, phase)) {
-                                    ok = mbar_wait(bfull0 + 8u * stage, phase, abort_flag, args.status, 8);
+                                ok = warp_wait(fb, phase, abort_flag, args.status, 4);
+                                if (!ok) break;
+                                if (PK) {
+                                    ok = warp_wait(bfull0 + 8u * stage, phase, abort_flag, args.status, 8);
                                     if (!ok) break;
                                 }
                                 // (the stage's operands were written by TMA, or by the expanding
