@@ -46,8 +46,15 @@ def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def headers() -> list[str]:
+    """Every header a source may include: a change of one rebuilds all objects,
+    which share its structures."""
+    return sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) +
+                  glob.glob(os.path.join(INCLUDE, "*.h")))
+
+
 def _deps() -> list[str]:
-    return sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h")) + [__file__]
+    return sources() + headers() + [__file__]
 
 
 def _stale(target: str, deps: list[str]) -> bool:
@@ -68,11 +75,10 @@ def build(force: bool = False, verbose: bool = False, extra_flags: list[str] | N
     os.makedirs(build_dir, exist_ok=True)
     nvcc = _nvcc()
     extra = list(extra_flags or []) + (["-DFASTID_DEBUG"] if debug else [])
-    headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
 
     def compile_one(src: str) -> str:
         obj = os.path.join(build_dir, os.path.basename(src)[:-3] + ".o")
-        if force or _stale(obj, [src, __file__] + headers):
+        if force or _stale(obj, [src, __file__] + headers()):
             cmd = [nvcc, *ARCH, *NVCC_FLAGS, *extra, "-c", src, "-o", obj]
             if verbose:
                 print(" ".join(cmd), file=sys.stderr)
