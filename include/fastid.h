@@ -301,8 +301,9 @@ fastid_status fastid_compare(fastid_ctx *ctx, const fastid_refdb *db, const uint
  *              block to the FP8 operand, which FASTID_FORM_TENSOR then reads).
  *              Every other case reads each block in the context's form: plain,
  *              FP8 expanded on chip, or FP4 (also FASTID_FORM_AUTO) -- for more
- *              than 128 queries through an FP4 operand built per block where
- *              the device has the memory, else expanded on chip.
+ *              than 128 queries through an FP4 operand built per block, where
+ *              both blocks' operands are at most a quarter of the device's
+ *              free memory, else expanded on chip.
  *  block_refs  largest block (>= 1; the first blocks are smaller, from
  *              block_refs / 8 doubling, so that the first comparison starts
  *              early).  Two blocks are on the device at once, each holding
@@ -310,7 +311,8 @@ fastid_status fastid_compare(fastid_ctx *ctx, const fastid_refdb *db, const uint
  *              the tensor form, its FP8 operand (n_loci rounded up to 128
  *              bytes per reference) or FP4 operand (n_loci rounded up to 256,
  *              half a byte each) or, for the plain form and forms expanded on
- *              chip, padded rows and popcounts.
+ *              chip, padded rows and popcounts.  The context keeps that
+ *              memory for its later calls until fastid_destroy.
  *  The other arguments are those of fastid_topk.  Stream-ordered: the call
  *  enqueues the copies and kernels and returns without waiting for them.
  * Errors: EINVAL, ENOMEM, ECUDA.

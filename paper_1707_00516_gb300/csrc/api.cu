@@ -520,14 +520,16 @@ struct TensorPrep {
 
 enum ExtraKind { EXTRA_NONE, EXTRA_TOPK };
 
-// run_s, run_i: running lists whose k-th scores start the shared cuts, or NULL.
-// op (an operand other than OP_PLAIN): FP8 or FP4 operands; packed rows
-// expanded on chip are unpaired, and their FP8 queries are encoded at half
-// scale to match the expanded 2.0.
-fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint64_t *q, int64_t ld_q, int64_t n_q,
-                             const uint8_t *modes, cudaStream_t s, Scratch &scr, ExtraKind ek, int64_t karg,
-                             size_t *extra_off, TensorPrep *tp, int op, const uint32_t *run_s = nullptr,
-                             const int64_t *run_i = nullptr) {
+// Places in a call's scratch.
+struct TensorOffsets {
+    size_t a, qconst, gcut, extra, bytes;
+};
+
+// A call's schedule and scratch (the host side of prepare_tensor).  op (an
+// operand other than OP_PLAIN): FP8 or FP4 operands; packed rows expanded on
+// chip are unpaired.
+fastid_status shape_tensor(fastid_ctx *ctx, const fastid_refdb *db, int64_t n_q, ExtraKind ek, int64_t karg, int op,
+                           TensorPrep *tp, TensorOffsets *at) {
     TcLaunch &L = tp->L;
     memset(&L, 0, sizeof L);
     const bool pk = op_packed(op), f4 = op_f4(op);
@@ -551,20 +553,45 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
     tp->n_ctas = (int64_t)L.n_groups * (L.pair ? 2 : 1);
     size_t extra = 0;
     if (ek == EXTRA_TOPK) extra = (size_t)L.n_slots * tensor_tile_q() * (size_t)karg * 8;
-    Carver cv;
-    size_t o_a = cv.take<uint8_t>((size_t)n_q_pad * kbytes);
-    size_t o_c = cv.take<float>((size_t)n_q_pad);
     if (ek == EXTRA_TOPK) plan_pub(L, 0, (int32_t)karg);
-    size_t o_g = cv.take<int32_t>(ek == EXTRA_TOPK ? (size_t)n_q_pad * (1 + L.n_pub[0]) : 0);
-    *extra_off = cv.take<uint8_t>(extra);
-    FASTID_CUDA(ctx, scr.alloc(cv.off));
-    const SharedCut cut{ek == EXTRA_TOPK ? at<int32_t>(scr.p, o_g) : nullptr, run_s, run_i, (int32_t)karg, n_q_pad,
-                        L.n_pub[0]};
-    uint8_t *a = at<uint8_t>(scr.p, o_a);
-    float *qconst = at<float>(scr.p, o_c);
+    Carver cv;
+    at->a = cv.take<uint8_t>((size_t)n_q_pad * kbytes);
+    at->qconst = cv.take<float>((size_t)n_q_pad);
+    at->gcut = cv.take<int32_t>(ek == EXTRA_TOPK ? (size_t)n_q_pad * (1 + L.n_pub[0]) : 0);
+    at->extra = cv.take<uint8_t>(extra);
+    at->bytes = cv.off;
+    L.n_panels = 1;
+    L.n_refs[0] = db->n_refs;
+    L.n_q[0] = n_q;
+    L.n_rt[0] = n_rt;
+    L.kpad[0] = kbytes;
+    L.gcut_ld[0] = n_q_pad;
     // spread the input queries over every tile of the operand (see
     // spread_row_to_query)
-    const int64_t spread = n_q_pad / tensor_tile_q();
+    L.qspread[0] = (int32_t)(n_q_pad / tensor_tile_q());
+    return FASTID_OK;
+}
+
+// run_s, run_i: running lists whose k-th scores start the shared cuts, or NULL.
+// FP8 queries over packed rows are encoded at half scale to match the expanded
+// 2.0.
+fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint64_t *q, int64_t ld_q, int64_t n_q,
+                             const uint8_t *modes, cudaStream_t s, Scratch &scr, ExtraKind ek, int64_t karg,
+                             size_t *extra_off, TensorPrep *tp, int op, const uint32_t *run_s = nullptr,
+                             const int64_t *run_i = nullptr) {
+    TensorOffsets o;
+    fastid_status st = shape_tensor(ctx, db, n_q, ek, karg, op, tp, &o);
+    if (st) return st;
+    TcLaunch &L = tp->L;
+    const bool pk = L.pk != 0, f4 = L.f4 != 0;
+    const int64_t n_q_pad = L.gcut_ld[0], spread = L.qspread[0];
+    const int32_t kbytes = L.kpad[0];
+    *extra_off = o.extra;
+    FASTID_CUDA(ctx, scr.alloc(o.bytes));
+    const SharedCut cut{ek == EXTRA_TOPK ? at<int32_t>(scr.p, o.gcut) : nullptr, run_s, run_i, (int32_t)karg, n_q_pad,
+                        L.n_pub[0]};
+    uint8_t *a = at<uint8_t>(scr.p, o.a);
+    float *qconst = at<float>(scr.p, o.qconst);
     if (f4)
         FASTID_CUDA(ctx, launch_queries_e2m1(q, ld_q, n_q, db->n_words64, db->n_loci, modes, n_q_pad, kbytes, a,
                                              qconst, spread, cut, s));
@@ -573,19 +600,12 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
                                              qconst, pk, spread, cut, s));
     count_launches(ctx, 1);
     FASTID_CUDA(ctx, make_operand_map(&L.map_a[0], a, n_q_pad, kbytes, tensor_tile_q()));
-    L.n_panels = 1;
     if (f4)
         L.map_b[0] = pk ? db->map_p4 : L.pair ? db->map_b4_half : db->map_b4;
     else
         L.map_b[0] = pk ? db->map_p : L.pair ? db->map_b_half : db->map_b;
-    L.n_refs[0] = db->n_refs;
-    L.n_q[0] = n_q;
-    L.n_rt[0] = n_rt;
-    L.kpad[0] = kbytes;
     L.qconst[0] = qconst;
     L.gcut[0] = cut.out;
-    L.gcut_ld[0] = n_q_pad;
-    L.qspread[0] = (int32_t)spread;
     L.status = ctx->dev_status;
     return FASTID_OK;
 }
@@ -888,6 +908,12 @@ Partition plain_partition(const fastid_ctx *ctx, int epi, int64_t n_q, int64_t n
     while ((128 >> t) != tile) ++t;
     const int kind = epi == EPI_TOPK ? 0 : epi == EPI_HITS ? 1 : 2;
     return make_partition(tile, n_q, n_pad / PL_TR, ctx->grid_plain[kind][t]);
+}
+
+size_t tensor_scratch_bytes(fastid_ctx *ctx, const fastid_refdb *db, int64_t n_q, int32_t k, int op) {
+    TensorPrep tp;
+    TensorOffsets o;
+    return shape_tensor(ctx, db, n_q, k > 0 ? EXTRA_TOPK : EXTRA_NONE, k, op, &tp, &o) == FASTID_OK ? o.bytes : 0;
 }
 
 MainTimer::MainTimer(fastid_ctx *c, cudaStream_t st) : ctx(c), s(st) {

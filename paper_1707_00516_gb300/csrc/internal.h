@@ -33,6 +33,9 @@ struct fastid_ctx {
     int grid_plain[3][fastid::PL_TILES] = {};  // plain CTAs resident at once: top-k, hits, scores; by tile height
     int grid_tensor = 0;
     int pair_clusters = 0;  // resident 2-CTA clusters of the paired tensor kernel (0: never pair)
+    // Most bytes that a streamed call's FP4 block operands may take; negative: a
+    // share of the device's free memory (stream.cu)
+    int64_t fp4_block_bytes = -1;
     std::string last_error;
     // profiling (fastid_profile)
     bool profile = false;
@@ -100,6 +103,18 @@ int pick_operand(int form, bool has_fp8, bool has_fp4, int64_t n_q, bool slots16
 // Work partition of a plain-form launch over n_pad padded references; its
 // query operand has n_qt * tile_q rows.
 Partition plain_partition(const fastid_ctx *ctx, int epi, int64_t n_q, int64_t n_pad);
+
+// Bytes of scratch that a comparison in a tensor form takes from the context's
+// pool: a top-k of depth k, or (k = 0) hits or full scores.  0 for a call that
+// has no schedule.
+size_t tensor_scratch_bytes(fastid_ctx *ctx, const fastid_refdb *db, int64_t n_q, int32_t k, int op);
+
+// Streamed calls: references of the block that follows one of `last` (0: of
+// the first), of at most `block`; and the most scratch that a call's
+// comparisons take, block after block (db: the row bytes of its blocks).
+int64_t stream_next_block(int64_t last, int64_t block);
+size_t stream_scratch_bytes(fastid_ctx *ctx, fastid_refdb db, int64_t n_refs, int64_t block, int64_t n_q, int32_t k,
+                            int op);
 
 // Argument checks of the top-k entry points (fastid_topk, fastid_topk_noalloc,
 // fastid_topk_accumulate): the shared query arguments, k, and the two output

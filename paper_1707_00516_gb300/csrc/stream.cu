@@ -128,18 +128,43 @@ fastid_status check_refs(fastid_ctx *ctx, const StreamRefs &r) {
     return FASTID_OK;
 }
 
-// Both slots' FP4 operands.  They take up to four times the packed rows'
-// memory, so where they do not fit -- or would leave too little for the
-// comparisons' own scratch (query operand and top-k lists), which is taken
-// and given back here to see -- the call goes on over packed rows: false,
-// nothing held.
-bool take_fp4(StreamState &st, int64_t cap, int64_t n_q, int32_t k) {
-    cudaError_t e = cudaSuccess;
-    const size_t kb = (size_t)st.slot[0].db.kbytes4;
-    for (Slot &sl : st.slot) sl.db.fp4 = static_cast<uint8_t *>(st.take((size_t)cap * kb, e));
-    const size_t tiles = (size_t)rup(n_q, 2 * TC_TILE_Q) / TC_TILE_Q;
-    void *probe = st.take(tiles * TC_TILE_Q * (kb + 4) + (4 * (size_t)st.ctx->grid_tensor + 4 * tiles) * TC_TILE_Q * k * 8,
-                          e);
+// Whether a call may take `operands` bytes for its blocks' FP4 operands beside
+// the comparisons' `scratch`.  The operands take up to four times the packed
+// rows' memory, and the context's pool keeps what it has taken: so they come out
+// of memory that the pool already holds unused, or are at most a quarter of
+// that and the device's free memory together -- enough for blocks of 4M
+// references at N = 2048 (8.6 GB) on an otherwise idle GPU, and the other
+// users of the device keep the rest.
+constexpr int FP4_FREE_SHARE = 4;
+
+bool fp4_allowed(fastid_ctx *ctx, size_t operands, size_t scratch) {
+    if (ctx->fp4_block_bytes >= 0) return operands <= (size_t)ctx->fp4_block_bytes;
+    uint64_t used = 0, reserved = 0;
+    size_t free_bytes = 0, total = 0;
+    cudaError_t e = cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used);
+    if (e == cudaSuccess) e = cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &reserved);
+    const size_t held = reserved > used ? (size_t)(reserved - used) : 0;
+    if (e == cudaSuccess && operands + scratch <= held) return true;
+    if (e == cudaSuccess) e = cudaMemGetInfo(&free_bytes, &total);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return operands <= (free_bytes + held) / FP4_FREE_SHARE;
+}
+
+// Both slots' FP4 operands, where they are allowed and fit together with the
+// comparisons' scratch (taken and given back here to see: each block's call
+// takes it again in stream order); else the call goes on over packed rows:
+// false, nothing held.
+bool take_fp4(StreamState &st, int64_t cap, size_t scratch) {
+    fastid_ctx *ctx = st.ctx;
+    const size_t operand = (size_t)cap * st.slot[0].db.kbytes4;
+    if (!fp4_allowed(ctx, 2 * operand, scratch)) return false;
+    uint64_t before = 0;
+    cudaError_t e = cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &before);
+    for (Slot &sl : st.slot) sl.db.fp4 = static_cast<uint8_t *>(st.take(operand, e));
+    void *probe = st.take(scratch, e);
     if (probe) cudaFreeAsync(probe, st.s);
     if (e == cudaSuccess) return true;
     cudaGetLastError();
@@ -147,13 +172,15 @@ bool take_fp4(StreamState &st, int64_t cap, int64_t n_q, int32_t k) {
         if (sl.db.fp4) cudaFreeAsync(sl.db.fp4, st.s);
         sl.db.fp4 = nullptr;
     }
+    cudaMemPoolTrimTo(ctx->pool, (size_t)before);  // (what the packed rows do not take over)
     return false;
 }
 
 // The block pipeline (see the top of this file).  `setup(st)` allocates the
 // entry point's own buffers (take_extra) and enqueues its initial work on the
 // caller's stream; `compare(b, db, r0)` enqueues block b's comparison of
-// db (references r0 .. r0 + db.n_refs - 1) there.
+// db (references r0 .. r0 + db.n_refs - 1) there: a top-k of depth k, or hits
+// (k = 0).
 template <class Setup, class Compare>
 fastid_status stream_blocks(fastid_ctx *ctx, const StreamRefs &R, int64_t n_q, int32_t k, cudaStream_t s, Setup setup,
                             Compare compare) {
@@ -194,7 +221,7 @@ fastid_status stream_blocks(fastid_ctx *ctx, const StreamRefs &R, int64_t n_q, i
     if (e != cudaSuccess) return scuda(ctx, e, "block buffers");
     fastid_status rs = setup(st);
     if (rs != FASTID_OK) return rs;
-    if (f4) f4 = take_fp4(st, cap, n_q, k);
+    if (f4) f4 = take_fp4(st, cap, stream_scratch_bytes(ctx, st.slot[0].db, R.n_refs, block, n_q, k, op));
     const bool rows = !tensor && !f4;
     for (Slot &sl : st.slot) {
         fastid_refdb &db = sl.db;
@@ -220,13 +247,13 @@ fastid_status stream_blocks(fastid_ctx *ctx, const StreamRefs &R, int64_t n_q, i
         (e = cudaStreamWaitEvent(st.expand, st.ready, 0)))
         return scuda(ctx, e, "stream ordering");
 
-    int64_t r0 = 0, next = std::max<int64_t>(std::min<int64_t>(block, ROW_ALIGN), block / 8);
+    int64_t r0 = 0, next = stream_next_block(0, block);
     for (int64_t b = 0; r0 < R.n_refs; ++b) {
         const int i = (int)(b & 1);
         Slot &sl = st.slot[i];
         fastid_refdb &db = sl.db;
         const int64_t n = std::min<int64_t>(next, R.n_refs - r0);
-        next = std::min<int64_t>(block, 2 * next);
+        next = stream_next_block(next, block);
         // copy: staging[i] is free once block b - 2 was expanded from it
         if (b >= 2 && (e = cudaStreamWaitEvent(st.copy, st.expanded[i], 0))) return scuda(ctx, e, "wait");
         e = cudaMemcpy2DAsync(sl.staging, (size_t)n_words * 8, R.host + r0 * R.ld_words, (size_t)R.ld_words * 8,
@@ -267,6 +294,33 @@ fastid_status stream_blocks(fastid_ctx *ctx, const StreamRefs &R, int64_t n_q, i
 }
 
 }  // namespace
+
+namespace fastid {
+
+int64_t stream_next_block(int64_t last, int64_t block) {
+    return last == 0 ? std::max<int64_t>(std::min<int64_t>(block, ROW_ALIGN), block / 8)
+                     : std::min<int64_t>(block, 2 * last);
+}
+
+size_t stream_scratch_bytes(fastid_ctx *ctx, fastid_refdb db, int64_t n_refs, int64_t block, int64_t n_q, int32_t k,
+                            int op) {
+    size_t most = 0;
+    int64_t next = 0, last = 0;
+    for (int64_t r0 = 0; r0 < n_refs; r0 += db.n_refs) {
+        next = stream_next_block(next, block);
+        db.n_refs = std::min<int64_t>(next, n_refs - r0);
+        if (db.n_refs == last) {  // full blocks from here: on to the remainder
+            r0 += ((n_refs - r0) / last - 1) * last;
+            continue;
+        }
+        last = db.n_refs;
+        db.n_pad = rup(db.n_refs, ROW_ALIGN);
+        most = std::max(most, tensor_scratch_bytes(ctx, &db, n_q, k, op));
+    }
+    return most;
+}
+
+}  // namespace fastid
 
 extern "C" {
 
@@ -327,10 +381,10 @@ fastid_status fastid_compare_streamed(fastid_ctx *ctx, const uint64_t *refs_host
     int64_t n_blocks = 0;
     {
         const int64_t block = std::min<int64_t>(block_refs, n_refs);
-        int64_t r0 = 0, next = std::max<int64_t>(std::min<int64_t>(block, ROW_ALIGN), block / 8);
+        int64_t r0 = 0, next = stream_next_block(0, block);
         for (; r0 < n_refs; ++n_blocks) {
             r0 += std::min<int64_t>(next, n_refs - r0);
-            next = std::min<int64_t>(block, 2 * next);
+            next = stream_next_block(next, block);
         }
     }
     unsigned long long *count = nullptr, *snaps = nullptr;
@@ -356,7 +410,7 @@ fastid_status fastid_compare_streamed(fastid_ctx *ctx, const uint64_t *refs_host
         ctx->launches += r0 != 0 && capacity > 0 ? 2 : 1;
         return FASTID_OK;
     };
-    if ((rs = stream_blocks(ctx, R, n_q, 1, s, setup, compare)) != FASTID_OK) return rs;
+    if ((rs = stream_blocks(ctx, R, n_q, 0, s, setup, compare)) != FASTID_OK) return rs;
     cudaError_t e = launch_hits_finish(count, capacity, n_q, n_refs, hit_q_dev, hit_r_dev, hit_score_dev, hit_count_dev,
                                        ctx->dev_status, s);
     if (e != cudaSuccess) return scuda(ctx, e, "hit list finish");
