@@ -622,7 +622,8 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
 //   64, 32        212 / 142            268 / 243    349 / 381    1404 / 1961
 // and the same at N = 512, 1024 and 4096 for as many bytes of packed rows
 // (256 bytes a row at N = 2048).
-bool use_few(int op, const fastid_refdb *db, int64_t n_q, int32_t k, FewShape *S) {
+bool use_few(const fastid_ctx *ctx, int op, const fastid_refdb *db, int64_t n_q, int32_t k, FewShape *S) {
+    if (ctx->few_rule != 0) return ctx->few_rule > 0 && op == OP_FP4_PACKED && few_shape(n_q, db->n_loci, k, S);
     const int64_t bytes = db->n_refs * db->ld64 * 8;
     if (n_q > 32 && bytes < (n_q <= 48 ? 320ll << 20 : 640ll << 20)) return false;
     return op == OP_FP4_PACKED && few_shape(n_q, db->n_loci, k, S);
@@ -755,7 +756,7 @@ fastid_status fastid_topk(fastid_ctx *ctx, const fastid_refdb *db, const uint64_
     FASTID_CUDA(ctx, cudaSetDevice(ctx->device));
     cudaStream_t s = (cudaStream_t)stream;
     FewShape few;
-    if (use_few(tensor, db, n_q, k, &few))
+    if (use_few(ctx, tensor, db, n_q, k, &few))
         return topk_few(ctx, db, few, queries_dev, ld_q, n_q, modes_dev, k, threshold, out_scores_dev, out_idx_dev,
                         false, 0, s);
     Scratch scr(ctx, s);
@@ -810,7 +811,7 @@ fastid_status fastid_topk_accumulate(fastid_ctx *ctx, const fastid_refdb *db, in
     FASTID_CUDA(ctx, cudaSetDevice(ctx->device));
     cudaStream_t s = (cudaStream_t)stream;
     FewShape few;
-    if (use_few(op, db, n_q, k, &few))
+    if (use_few(ctx, op, db, n_q, k, &few))
         return topk_few(ctx, db, few, queries_dev, ld_q, n_q, modes_dev, k, threshold, run_scores_dev, run_idx_dev,
                         true, ref_offset, s);
     Scratch scr(ctx, s);

@@ -1,5 +1,6 @@
 // What tests set in a context that the C ABI does not offer; compiled against
 // the library's internal header and called with a context's handle.
+#include "few.h"
 #include "internal.h"
 
 extern "C" {
@@ -7,6 +8,16 @@ extern "C" {
 // Most bytes that a streamed call's FP4 block operands may take (negative: the
 // library's own rule).
 void hook_fp4_block_bytes(fastid_ctx *ctx, int64_t bytes) { ctx->fp4_block_bytes = bytes; }
+
+// Top-k calls over packed rows: 0 the library's rule, 1 the few-query form
+// wherever it fits, -1 never.
+void hook_few_rule(fastid_ctx *ctx, int32_t rule) { ctx->few_rule = rule; }
+
+// Packed stages of the few-query form for such a call; 0: it does not fit.
+int32_t hook_few_stages(int64_t n_q, int32_t n_loci, int32_t k) {
+    fastid::FewShape S;
+    return fastid::few_shape(n_q, n_loci, k, &S) ? S.stages : 0;
+}
 
 // Row bytes of an FP4 operand.
 int32_t hook_kbytes4(int32_t n_loci) { return fastid::tensor_kbytes4(n_loci); }
