@@ -610,23 +610,12 @@ fastid_status prepare_tensor(fastid_ctx *ctx, const fastid_refdb *db, const uint
     return FASTID_OK;
 }
 
-// Which top-k calls over packed rows take the few-query form (few.cu).  It is
-// always the faster up to 32 queries; with more its lists take longer to fill
-// than the tensor kernel's, which a short database does not repay.  Measured
-// (us, few-query form against the tensor kernel over packed rows):
-//   queries, k    N = 2048 x 500,000   1.5M         3M           20M
-//   32, 10        84 / 99              128 / 189    200 / 315    1065 / 1810
-//   48, 10        107 / 99             148 / 189    221 / 315    1128 / 1810
-//   48, 32        163 / 142            236 / 243    301 / 381    1206 / 1961
-//   64, 10        127 / 99             175 / 189    264 / 315    1320 / 1810
-//   64, 32        212 / 142            268 / 243    349 / 381    1404 / 1961
-// and the same at N = 512, 1024 and 4096 for as many bytes of packed rows
-// (256 bytes a row at N = 2048).
+// Which top-k calls over packed rows take the few-query form (few.cu): where it
+// fits and pays (few_pays), or as the context says.
 bool use_few(const fastid_ctx *ctx, int op, const fastid_refdb *db, int64_t n_q, int32_t k, FewShape *S) {
-    if (ctx->few_rule != 0) return ctx->few_rule > 0 && op == OP_FP4_PACKED && few_shape(n_q, db->n_loci, k, S);
-    const int64_t bytes = db->n_refs * db->ld64 * 8;
-    if (n_q > 32 && bytes < (n_q <= 48 ? 320ll << 20 : 640ll << 20)) return false;
-    return op == OP_FP4_PACKED && few_shape(n_q, db->n_loci, k, S);
+    if (op != OP_FP4_PACKED || ctx->few_rule < 0) return false;
+    if (ctx->few_rule == 0 && !few_pays(n_q, k, db->n_refs, db->ld64 * 8)) return false;
+    return few_shape(n_q, db->n_loci, k, S);
 }
 
 // Few-query launch of a top-k call (few.cu) over packed rows.

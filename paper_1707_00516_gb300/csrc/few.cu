@@ -743,6 +743,41 @@ bool few_shape(int64_t n_q, int32_t n_loci, int32_t k, FewShape *S) {
     return true;
 }
 
+// The tensor kernel takes one query as it takes 128, and its lists fill faster;
+// this form streams the rows faster, starts its cuts from a sample, and takes
+// longer with every query and with k.  So up to 8 queries it is never the slower
+// by more than 3 us, and with more it needs a database long enough to repay its
+// lists, and rows wider than 256 bytes (N = 2048) one long enough to repay four
+// rounds of samples (seed kernel).  Above k = 16 the tensor kernel's lists are
+// the slower 32-slot ones.  Measured (fastid_topk, us, this form / the tensor
+// kernel over packed rows; MiB of packed rows, N = 2048 unless named):
+//   queries, k      0.5     24        61         122        244        366        659
+//    8, 10        24/31    35/46    44/62      56/90      81/132     106/178    169/277
+//   16, 1         26/22    37/33    43/50      56/78      82/122     109/166    171/266
+//   16, 10        29/32    43/48    51/62      65/90      87/134     114/179    175/279
+//   32, 1         32/23    45/33    52/52      63/80      84/123     111/168    173/268
+//   32, 10        37/33    53/48    67/66      83/92      101/136    126/182    187/281
+//   32, 32        51/54    62/77    91/98      117/128    150/172    166/223    225/329
+//   48, 1         40/23    53/35    58/52      73/81      87/124     117/168    181/268
+//   48, 10        45/33    64/48    83/65      101/93     123/137    144/182    207/281
+//   48, 32        64/54    82/77    124/97     159/128    204/173    228/223    282/328
+//   64, 1         46/24    60/35    65/54      76/80      101/124    137/168    212/269
+//   64, 10        53/33    84/48    102/66     127/95     148/137    178/183    251/282
+//   64, 32        78/54    107/77   159/98     205/128    246/175    270/224    334/329
+//   16, 10, N = 8192       57/45               90/84                 (488: 165/212)
+//   32, 32, N = 8192       68/68               115/109               (488: 187/242)
+// and N = 200 and 512 as N = 2048 for as many bytes.  (With one line for every k,
+// and none up to 32 queries, 32 queries of k = 1 took 36 us over 1000 references
+// where the tensor kernel takes 23 and took 29 before its queues.)
+bool few_pays(int64_t n_q, int32_t k, int64_t n_refs, int64_t row_bytes) {
+    if (n_q <= 8) return true;
+    // the shortest database, KiB of packed rows: up to 16, 32, 48, 64 queries; k up to 4, up to 16, above
+    constexpr int64_t least[4][3] = {
+        {32 << 10, 256, 0}, {48 << 10, 48 << 10, 256}, {112 << 10, 224 << 10, 384 << 10}, {224 << 10, 448 << 10, 640 << 10}};
+    const int64_t wide = k <= 16 && row_bytes > 256 ? (row_bytes - 256) * 200 : 0;
+    return n_refs * row_bytes >= (least[std::min<int64_t>((n_q - 1) / 16, 3)][k <= 4 ? 0 : k <= 16 ? 1 : 2] + wide) << 10;
+}
+
 cudaError_t launch_few_seed(const FewLaunch &L, const FewShape &S, cudaStream_t s) {
     // At most a sixteenth of the references.  With up to 8 queries the seeds
     // are on the call's critical path and one round is enough (one query over

@@ -15,6 +15,10 @@ struct FewShape {
 // and at least four packed stages fit an SM's shared memory.
 bool few_shape(int64_t n_q, int32_t n_loci, int32_t k, FewShape *S);
 
+// Whether it is the faster for a call that it fits: k deep, over n_refs packed
+// rows of row_bytes.
+bool few_pays(int64_t n_q, int32_t k, int64_t n_refs, int64_t row_bytes);
+
 struct FewLaunch {
     const uint64_t *q;  // packed queries
     int64_t ld_q, n_q;

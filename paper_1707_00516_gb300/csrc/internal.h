@@ -34,7 +34,7 @@ struct fastid_ctx {
     int grid_tensor = 0;
     int pair_clusters = 0;  // resident 2-CTA clusters of the paired tensor kernel (0: never pair)
     // Top-k calls over packed rows that the few-query form fits: 0 take it where
-    // use_few says so (api.cu), 1 always, -1 never
+    // few_pays says so (few.h), 1 always, -1 never
     int few_rule = 0;
     // Most bytes that a streamed call's FP4 block operands may take; negative: a
     // share of the device's free memory (stream.cu)

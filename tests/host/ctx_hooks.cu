@@ -19,6 +19,11 @@ int32_t hook_few_stages(int64_t n_q, int32_t n_loci, int32_t k) {
     return fastid::few_shape(n_q, n_loci, k, &S) ? S.stages : 0;
 }
 
+// The library's rule for it: k deep, over n_refs packed rows of row_bytes.
+int32_t hook_few_pays(int64_t n_q, int32_t k, int64_t n_refs, int64_t row_bytes) {
+    return fastid::few_pays(n_q, k, n_refs, row_bytes);
+}
+
 // Row bytes of an FP4 operand.
 int32_t hook_kbytes4(int32_t n_loci) { return fastid::tensor_kbytes4(n_loci); }
 }
