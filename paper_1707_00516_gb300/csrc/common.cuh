@@ -44,6 +44,7 @@ struct Partition {
     int32_t grid;      // G
     int32_t max_seg;   // max query-tile segments per CTA
     int32_t tile_q;    // queries a tile
+    int32_t fills;     // the CTAs take every place on the GPU (see launch_plain)
 };
 
 __host__ __device__ inline int64_t part_begin(const Partition &p, int64_t c) {
@@ -61,6 +62,7 @@ __host__ inline Partition make_partition(int32_t tile_q, int64_t n_q, int64_t n_
     if (g > p.n_units) g = p.n_units;
     if (g < 1) g = 1;
     p.grid = (int32_t)g;
+    p.fills = g >= grid_target ? 1 : 0;
     int64_t span = (p.n_units + g - 1) / g;
     p.max_seg = (int32_t)((span + n_rt - 1) / n_rt + 1);
     return p;

@@ -480,7 +480,13 @@ cudaError_t launch_plain(int epi, const uint32_t *refs32, const uint32_t *ref_no
     cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_dependent(fn, dim3((unsigned)part.grid), dim3(PL_THREADS), smem, s, a);
+    // Beside the query preparation only where the CTAs fill the GPU: fewer of
+    // them, launched while its blocks are still there, go two to an SM where those
+    // are not and leave other SMs idle (1000 queries x 1000 references, 64 CTAs,
+    // k = 10: 142 us beside it, 108 after it).
+    if (part.fills) return launch_dependent(fn, dim3((unsigned)part.grid), dim3(PL_THREADS), smem, s, a);
+    fn<<<(unsigned)part.grid, PL_THREADS, smem, s>>>(a);
+    return cudaGetLastError();
 }
 
 }  // namespace fastid

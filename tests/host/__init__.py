@@ -26,5 +26,6 @@ def ctx_hooks(tmp) -> ctypes.CDLL:
     lib.hook_few_rule.restype = None
     lib.hook_few_stages.argtypes = [ctypes.c_int64, ctypes.c_int32, ctypes.c_int32]
     lib.hook_few_pays.argtypes = [ctypes.c_int64, ctypes.c_int32, ctypes.c_int64, ctypes.c_int64]
+    lib.hook_plain_fills.argtypes = [ctypes.c_int32, ctypes.c_int32, ctypes.c_int64, ctypes.c_int64]
     lib.hook_kbytes4.argtypes = [ctypes.c_int32]
     return lib

@@ -24,6 +24,14 @@ int32_t hook_few_pays(int64_t n_q, int32_t k, int64_t n_refs, int64_t row_bytes)
     return fastid::few_pays(n_q, k, n_refs, row_bytes);
 }
 
+// Whether a plain launch's CTAs take every place of a GPU that holds `places`
+// of them.
+int32_t hook_plain_fills(int32_t places, int32_t tile_q, int64_t n_q, int64_t n_refs) {
+    const int64_t n_rt = (n_refs + fastid::ROW_ALIGN - 1) / fastid::ROW_ALIGN * (fastid::ROW_ALIGN / fastid::PL_TR);
+    const fastid::Partition p = fastid::make_partition(tile_q, n_q, n_rt, places);
+    return p.fills;
+}
+
 // Row bytes of an FP4 operand.
 int32_t hook_kbytes4(int32_t n_loci) { return fastid::tensor_kbytes4(n_loci); }
 }
