@@ -229,6 +229,10 @@ __global__ void hits_offset_kernel(const unsigned long long *__restrict__ snaps,
 // 2^21, whatever the count; the count kernel and four passes take ~53 us, half
 // of it the global atomics of the next counts: a kernel of its own for those
 // would cost as much.)
+// Up to RS_FEW hits the count kernel's first block sorts them itself, each
+// hit's place being the number of hits before it, and the passes have nothing
+// to do: their latencies alone (19 us for two hits, where the bitonic sort of a
+// small buffer took 3) were a third of a small call.
 constexpr int RS_BITS = 8;
 constexpr int RS_DIGITS = 1 << RS_BITS;
 constexpr int RS_THREADS = 1024;
@@ -236,6 +240,7 @@ constexpr int RS_ITEMS = 4;  // elements a thread
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
 constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_GROUPS = RS_THREADS / RS_DIGITS;
+constexpr int RS_FEW = 512;
 constexpr int RS_BLOCKS = 256;  // about what fits the GPU at once (two a SM); every block reads every block's counts
 
 __device__ __forceinline__ int64_t hits_live(const unsigned long long *count, int64_t capacity) {
@@ -251,12 +256,13 @@ __device__ __forceinline__ int rs_shift(int64_t n) {
 }
 static_assert(RS_TILE == 1 << 12, "rs_shift starts at one tile");
 
-// The true count to the caller, the overflow condition, and the first pass's digit counts.
+// The true count to the caller, the overflow condition, and the first pass's
+// digit counts -- or the sorted list, where the hits are few.
 __global__ void __launch_bounds__(RS_THREADS) hits_count_kernel(const unsigned long long *__restrict__ count,
                                                                 int64_t capacity, int64_t *__restrict__ count_out,
                                                                 uint32_t *__restrict__ status,
-                                                                const int64_t *__restrict__ hq,
-                                                                const int64_t *__restrict__ hr, int r_bits,
+                                                                int64_t *__restrict__ hq, int64_t *__restrict__ hr,
+                                                                uint32_t *__restrict__ hs, int r_bits,
                                                                 uint32_t *__restrict__ table) {
     pdl_trigger();
     pdl_wait();
@@ -269,6 +275,26 @@ __global__ void __launch_bounds__(RS_THREADS) hits_count_kernel(const unsigned l
     const int sh = rs_shift(n);
     const int64_t b0 = (int64_t)blockIdx.x << sh;
     if (b0 >= n) return;
+    if (n <= RS_FEW) {  // (one block)
+        __shared__ uint64_t keys[RS_FEW];
+        const int i = threadIdx.x, live = (int)n;
+        uint64_t key = 0;
+        uint32_t score = 0;
+        if (i < live) {
+            key = ((uint64_t)hq[i] << r_bits) | (uint64_t)hr[i];
+            score = hs[i];
+            keys[i] = key;
+        }
+        __syncthreads();
+        if (i >= live) return;
+        int at = 0;
+#pragma unroll 8
+        for (int j = 0; j < live; ++j) at += keys[j] < key || (keys[j] == key && j < i);
+        hq[at] = (int64_t)(key >> r_bits);
+        hr[at] = (int64_t)(key & ((1ull << r_bits) - 1ull));
+        hs[at] = score;
+        return;
+    }
     __shared__ uint32_t cnt[RS_DIGITS];
     if (threadIdx.x < RS_DIGITS) cnt[threadIdx.x] = 0;
     __syncthreads();
@@ -294,6 +320,7 @@ __global__ void __launch_bounds__(RS_THREADS)
     pdl_trigger();
     pdl_wait();
     const int64_t n = hits_live(count, capacity);
+    if (n <= RS_FEW) return;  // sorted already
     const int sh = rs_shift(n);
     const int64_t b0 = (int64_t)blockIdx.x << sh, b1 = min(n, b0 + ((int64_t)1 << sh));
     if (b0 >= n) return;
@@ -497,7 +524,7 @@ cudaError_t launch_hits_finish(void *aux, int64_t capacity, int64_t n_q, int64_t
     const unsigned grid = (unsigned)std::max<int64_t>(1, nb);
     const dim3 blocks(grid), threads(RS_THREADS);
     cudaError_t e = launch_dependent(hits_count_kernel, blocks, threads, 0, s, count, capacity, count_out, status, hit_q,
-                                     hit_r, r_bits, table);
+                                     hit_r, hit_score, r_bits, table);
     if (capacity == 0) return e;
     uint64_t *hk = reinterpret_cast<uint64_t *>(hit_q);
     for (int p = 0; p < passes && e == cudaSuccess; ++p) {
