@@ -61,7 +61,7 @@ class Searcher:
         B.fastid_pack(self.ctx, src_alleles, n_loci, src_packed)
         q = self._buf("queries", (n_q, w), torch.int64)
         B.fastid_mix(self.ctx, src_packed, w, offsets, q)
-        return q
+        return q.detach()  # the caller's own tensor over the buffer: a change of its shape is not the buffer's
 
     def tune_form(self, db: B.RefDB, queries: torch.Tensor, modes: torch.Tensor, k: int,
                   threshold: int = B.NO_THRESHOLD, tuner=None) -> int:
