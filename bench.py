@@ -288,10 +288,11 @@ def run_reference(args, w):
 # ----------------------------------------------------------------------------
 
 def kernel_source_hash(form: str) -> str:
-    """Hash of the kernel's source with comments and whitespace removed, so
-    that edits to comments alone keep the recorded ncu figures valid."""
+    """Hash of the kernel's source and the headers it includes, with comments
+    and whitespace removed, so that edits to comments alone keep the recorded
+    ncu figures valid."""
     h = hashlib.sha256()
-    for f in ("plain.cu" if form == "plain" else "tensor.cu", "common.cuh"):
+    for f in ("plain.cu", "common.cuh", "keys.cuh") if form == "plain" else ("tensor.cu", "common.cuh", "tc_ptx.cuh"):
         with open(os.path.join(ROOT, "paper_1707_00516_gb300", "csrc", f)) as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
