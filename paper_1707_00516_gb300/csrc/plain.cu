@@ -15,7 +15,7 @@
 //
 // CTA tile: 128 references x TQ queries, 256 threads, each thread owns 8
 // references (rows tr + 16 i) and JQ = TQ / 16 queries (rows tq + 16 j) of the
-// tile; two CTAs an SM at TQ = 128, more below.  TQ is 128, 64, 32 or 16, the
+// tile; two CTAs an SM at TQ = 128 and 64, three below.  TQ is 128, 64, 32 or 16, the
 // one that pads the call's queries least (plain_tile_q): a tile costs its full
 // height whatever part of it is queries.
 // The grid is persistent: CTA c walks the units [c U / G, (c+1) U / G) of the

@@ -47,8 +47,11 @@ constexpr int TC_BM = 128;          // queries per tile
 constexpr int TC_BK = 128;          // loci (bytes) per stage
 constexpr int TC_THREADS = 192;     // producer, MMA issuer, 4 epilogue warps (a second set: 128 more)
 // PK: warps expanding packed references, after the 6 others.  Blocks of 257 to
-// 384 threads get at most 168 registers a thread, which the 16-slot top-k
-// fits (4 expanding warps) and the 32-slot one does not (2).
+// 384 threads get at most 168 registers a thread.  The 16-slot top-k runs with
+// that (4 expanding warps), its queues spilling 92 (FP8) and 100 (FP4) bytes a
+// thread: without queues nothing spilled and it was slower everywhere (96
+// queries, N = 2048, k = 10, FP4, us: 20,000 references 83 -> 35, 500,000 211 ->
+// 96, 2M 363 -> 225, 20M 1942 -> 1809).  The 32-slot one does not fit (2 warps).
 __host__ __device__ constexpr int pk_threads(int km) { return km == 16 ? 128 : 64; }
 constexpr uint32_t TC_A_BYTES = TC_BM * TC_BK;  // 16 KB
 // Packed reference stage of PK launches: BN rows of the stage's loci (128
