@@ -291,10 +291,14 @@ def kernel_source_hash(form: str) -> str:
     """Hash of the kernel's source and the headers it includes, with comments
     and whitespace removed, so that edits to comments alone keep the recorded
     ncu figures valid."""
+    csrc = os.path.join(ROOT, "paper_1707_00516_gb300", "csrc")
     h = hashlib.sha256()
-    for f in ("plain.cu", "common.cuh", "keys.cuh") if form == "plain" else ("tensor.cu", "common.cuh", "tc_ptx.cuh"):
-        with open(os.path.join(ROOT, "paper_1707_00516_gb300", "csrc", f)) as fh:
+    files = ["plain.cu" if form == "plain" else "tensor.cu", "common.cuh"]
+    for f in files:
+        with open(os.path.join(csrc, f)) as fh:
             src = fh.read()
+        files += [g for g in re.findall(r'#include "([^"]+)"', src)
+                  if g not in files and os.path.exists(os.path.join(csrc, g))]
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
         src = re.sub(r"//[^\n]*", " ", src)
         h.update(" ".join(src.split()).encode())
