@@ -29,7 +29,7 @@ class Searcher:
         B.fastid_set_form(self.ctx, form)
         self._pinned: dict[str, torch.Tensor] = {}
         self._devbuf: dict[str, torch.Tensor] = {}
-        self._devview: dict[str, tuple] = {}  # a buffer's last shape and its view
+        self._devview: dict[str, torch.Tensor] = {}  # a buffer's last view
 
     # ---- database ------------------------------------------------------
     def load_refs_packed(self, packed: torch.Tensor, n_loci: int, flags: int = 0) -> B.RefDB:
@@ -53,7 +53,11 @@ class Searcher:
 
     # ---- queries ---------------------------------------------------------
     def build_queries(self, src_alleles: torch.Tensor, offsets: torch.Tensor, n_loci: int) -> torch.Tensor:
-        """Pack contributor rows and OR each group into one query profile."""
+        """Pack contributor rows and OR each group into one query profile.
+
+        The result lies in the searcher's buffer: the next call overwrites it,
+        and may return the same tensor object.
+        """
         n_src = src_alleles.shape[0]
         n_q = offsets.numel() - 1
         w = words64(n_loci)
@@ -61,7 +65,7 @@ class Searcher:
         B.fastid_pack(self.ctx, src_alleles, n_loci, src_packed)
         q = self._buf("queries", (n_q, w), torch.int64)
         B.fastid_mix(self.ctx, src_packed, w, offsets, q)
-        return q.detach()  # the caller's own tensor over the buffer: a change of its shape is not the buffer's
+        return q
 
     def tune_form(self, db: B.RefDB, queries: torch.Tensor, modes: torch.Tensor, k: int,
                   threshold: int = B.NO_THRESHOLD, tuner=None) -> int:
@@ -117,17 +121,22 @@ class Searcher:
 
     # ---- host in, host out ---------------------------------------------
     def _buf(self, name, shape, dtype):
+        # The last view again, if it is one of this shape still: callers have
+        # had it, and may have changed its shape in place.  (A new view each time
+        # costs small calls 8 us, these checks 1.5: 2048 queries of 1501 loci 22 and
+        # 15.3 us a call, 13.7 with neither.)
         shape = tuple(shape)
-        last = self._devview.get(name)
-        if last is not None and last[0] == shape and last[1] == dtype:
-            return last[2]
         t = self._devbuf.get(name)
+        v = self._devview.get(name)
+        if (v is not None and v.shape == shape and v.dtype == dtype and v.is_contiguous()
+                and v.data_ptr() == t.data_ptr()):
+            return v
         n = math.prod(shape)
         if t is None or t.numel() < n or t.dtype != dtype:
             t = torch.empty(max(n, 1), dtype=dtype, device=self.device)
             self._devbuf[name] = t
         v = t[:n].view(shape)
-        self._devview[name] = (shape, dtype, v)
+        self._devview[name] = v
         return v
 
     def _pin(self, name, arr: np.ndarray) -> torch.Tensor:
