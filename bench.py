@@ -551,9 +551,10 @@ def run_gpu(args, w):
 
 def run_streamed(args, w):
     """The workload with its references in pinned HOST memory, streamed
-    through the device in blocks by fastid_topk_streamed: FP4 over each
-    block's packed rows (the library's AUTO choice), or with --form fp8 each
-    block expanded to the FP8 operand, or fp8packed / plain over the rows."""
+    through the device in blocks by fastid_topk_streamed: each block expanded
+    to the FP4 operand (the library's AUTO choice above 128 queries), or with
+    --form fp8 to the FP8 operand, or fp4packed / fp8packed / plain over its
+    packed rows."""
     import torch
     from paper_1707_00516_gb300 import binding as B
     from paper_1707_00516_gb300 import peaks as P
@@ -564,7 +565,7 @@ def run_streamed(args, w):
     gen.build_gpu()
     build()
     probe = P.measure()
-    form = args.form if args.form in ("fp8", "fp8packed", "fp4packed", "plain") else "fp4packed"
+    form = args.form if args.form in FORMS else "fp4"
     s = Searcher(0, getattr(B, FORMS[form][0]))
     sflags = B.REFS_TENSOR if form == "fp8" else 0
     seed = gen.config_seed(w["cfg"])
