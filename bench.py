@@ -309,12 +309,12 @@ def kernel_source_hash(form: str) -> str:
 # (profiles/), keyed by form and workload, with the source hash it was taken
 # at.  A changed kernel reports null.
 NCU_TRAFFIC = {
-    # profiles/tensor_kernel_fp4_c3_2048x20M.md: dram__bytes_read.sum 25.01 GB + dram__bytes_write.sum 39.98 MB
-    "fp4/c3": (25.012413952e9 + 39.982848e6, "9f95518100d29482"),
-    # profiles/tensor_kernel_c3_2048x20M.md: dram__bytes_read.sum 76.39 GB + dram__bytes_write.sum 78.66 MB
-    "fp8/c3": (76.389554176e9 + 78.660864e6, "9f95518100d29482"),
-    # profiles/plain_kernel_c3_2048x20M.md: dram__bytes_read.sum 45.61 GB + dram__bytes_write.sum 28.82 MB
-    "plain/c3": (45.612705280e9 + 28.819456e6, "a0d17b3f0ba88167"),
+    # profiles/tensor_kernel_fp4_c3_2048x20M.md: dram__bytes_read.sum 29.92 GB + dram__bytes_write.sum 47.34 MB
+    "fp4/c3": (29.92e9 + 47.34e6, "3c5e48ecf01ea817"),
+    # profiles/tensor_kernel_c3_2048x20M.md: dram__bytes_read.sum 74.72 GB + dram__bytes_write.sum 84.18 MB
+    "fp8/c3": (74.72e9 + 84.18e6, "3c5e48ecf01ea817"),
+    # profiles/plain_kernel_c3_2048x20M.md: dram__bytes_read.sum 43.15 GB + dram__bytes_write.sum 28.98 MB
+    "plain/c3": (43.15e9 + 28.98e6, "7a613d2777771ec2"),
 }
 
 

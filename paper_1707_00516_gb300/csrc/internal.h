@@ -89,17 +89,17 @@ __host__ __device__ inline bool op_f4(int op) { return op == OP_FP4 || op == OP_
 // the packed rows expanded to FP4 on chip.  Measured with fastid_topk on 20M
 // references at N = 2048 (ms, k = 16 / k = 32):
 //   queries      FP4 copy    FP4 packed   FP8 copy    FP8 packed
-//   32-128       2.94/2.94   1.97/2.55    5.76/5.76   3.23/4.07
-//   256          3.58/3.58   3.75/4.99    6.68/6.69   6.25/8.04
-//   512          6.01/5.99   7.31/9.92    10.6/10.6   12.3/16.1
-//   2048         24.1/24.6   29.7/40.8    40.6/40.6   50.3/65.2
-// so the FP4 packed rows are never slower than an FP8 operand, and the FP4
-// copy wins from two query tiles on.
-// (Before the few-query form, few.cu, which takes up to 64 queries over the
-// packed rows in 1.04 to 1.40, and the cuts shared by a launch's slices.  One
-// query tile over a short database is even: 96 queries, k = 10 / 32, 500,000
-// references 111 / 147 us over the copy and 100 / 145 packed, 100,000 54 / 85
-// and 54 / 86.)
+//   32           2.92/2.94   1.09/1.12    5.69/5.71   3.01/3.94
+//   64           2.92/2.96   1.35/1.41    5.69/5.71   3.01/3.94
+//   100-128      2.93/2.98   1.81/1.96    5.69/5.71   3.02/3.96
+//   256          3.04/3.08   3.41/3.80    6.52/6.55   5.91/7.84
+//   512          5.38/5.45   6.58/7.50    10.5/10.6   11.7/15.6
+//   2048         18.3/18.3   25.6/30.3    38.1/37.7   46.5/63.1
+// so the FP4 packed rows (up to 64 queries the few-query form, few.cu) are never
+// slower than an FP8 operand, and the FP4 copy wins from two query tiles on.
+// One query tile over a short database is even: 96 queries, k = 10 / 32, 500,000
+// references 111 / 147 us over the copy and 96 / 135 packed, 100,000 54 / 85 and
+// 48 / 78.
 constexpr int64_t AUTO_FP4_PACKED_MAX_Q = 128;
 int pick_operand(int form, bool has_fp8, bool has_fp4, int64_t n_q, bool slots16 = true);
 
