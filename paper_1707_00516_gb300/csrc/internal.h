@@ -39,6 +39,7 @@ struct fastid_ctx {
     // Most bytes that a streamed call's FP4 block operands may take; negative: a
     // share of the device's free memory (stream.cu)
     int64_t fp4_block_bytes = -1;
+    size_t fp4_block_held = 0;  // the most that they have taken from the pool, which keeps it
     std::string last_error;
     // profiling (fastid_profile)
     bool profile = false;

@@ -128,29 +128,24 @@ fastid_status check_refs(fastid_ctx *ctx, const StreamRefs &r) {
     return FASTID_OK;
 }
 
-// Whether a call may take `operands` bytes for its blocks' FP4 operands beside
-// the comparisons' `scratch`.  The operands take up to four times the packed
-// rows' memory, and the context's pool keeps what it has taken: so they come out
-// of memory that the pool already holds unused, or are at most a quarter of
-// that and the device's free memory together -- enough for blocks of 4M
-// references at N = 2048 (8.6 GB) on an otherwise idle GPU, and the other
-// users of the device keep the rest.
+// Whether a call may take `operands` bytes for its blocks' FP4 operands.  They
+// take up to four times the packed rows' memory, and the context's pool keeps
+// what it has taken: so a call takes no more than an earlier one left in the
+// pool, or at most a quarter of that and the device's free memory together --
+// enough for blocks of 4M references at N = 2048 (8.6 GB) on an otherwise idle
+// GPU, and the other users of the device keep the rest.  (The pool's own
+// attributes may not be asked for while a stream is captured.)
 constexpr int FP4_FREE_SHARE = 4;
 
-bool fp4_allowed(fastid_ctx *ctx, size_t operands, size_t scratch) {
+bool fp4_allowed(fastid_ctx *ctx, size_t operands) {
     if (ctx->fp4_block_bytes >= 0) return operands <= (size_t)ctx->fp4_block_bytes;
-    uint64_t used = 0, reserved = 0;
+    if (operands <= ctx->fp4_block_held) return true;
     size_t free_bytes = 0, total = 0;
-    cudaError_t e = cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used);
-    if (e == cudaSuccess) e = cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &reserved);
-    const size_t held = reserved > used ? (size_t)(reserved - used) : 0;
-    if (e == cudaSuccess && operands + scratch <= held) return true;
-    if (e == cudaSuccess) e = cudaMemGetInfo(&free_bytes, &total);
-    if (e != cudaSuccess) {
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return operands <= (free_bytes + held) / FP4_FREE_SHARE;
+    return operands <= (free_bytes + ctx->fp4_block_held) / FP4_FREE_SHARE;
 }
 
 // Both slots' FP4 operands, where they are allowed and fit together with the
@@ -160,19 +155,27 @@ bool fp4_allowed(fastid_ctx *ctx, size_t operands, size_t scratch) {
 bool take_fp4(StreamState &st, int64_t cap, size_t scratch) {
     fastid_ctx *ctx = st.ctx;
     const size_t operand = (size_t)cap * st.slot[0].db.kbytes4;
-    if (!fp4_allowed(ctx, 2 * operand, scratch)) return false;
-    uint64_t before = 0;
-    cudaError_t e = cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &before);
+    if (!fp4_allowed(ctx, 2 * operand)) return false;
+    // (a captured call's memory is its graph's, not the pool's)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st.s, &capture) != cudaSuccess) cudaGetLastError();
+    cudaError_t e = cudaSuccess;
     for (Slot &sl : st.slot) sl.db.fp4 = static_cast<uint8_t *>(st.take(operand, e));
     void *probe = st.take(scratch, e);
     if (probe) cudaFreeAsync(probe, st.s);
-    if (e == cudaSuccess) return true;
+    if (e == cudaSuccess) {
+        if (capture == cudaStreamCaptureStatusNone) ctx->fp4_block_held = std::max(ctx->fp4_block_held, 2 * operand);
+        return true;
+    }
     cudaGetLastError();
     for (Slot &sl : st.slot) {
         if (sl.db.fp4) cudaFreeAsync(sl.db.fp4, st.s);
         sl.db.fp4 = nullptr;
     }
-    cudaMemPoolTrimTo(ctx->pool, (size_t)before);  // (what the packed rows do not take over)
+    if (capture == cudaStreamCaptureStatusNone) {  // give back what the pool holds unused: memory is short
+        cudaMemPoolTrimTo(ctx->pool, 0);
+        ctx->fp4_block_held = 0;
+    }
     return false;
 }
 
