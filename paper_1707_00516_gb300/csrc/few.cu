@@ -52,8 +52,8 @@
 // merging warps), so that few candidates ever arrive.
 //
 // Measured (fastid_topk, 20M references, N = 2048, us; the tensor kernel over
-// packed rows before -> this form): 1 query 1930 -> 1043, 48 mixtures 2000 ->
-// 1149, 64 at k = 32 2400 -> 1404.  HBM is the floor at 754; the SM's issue
+// packed rows before -> this form): 1 query 1930 -> 1043, 48 mixtures 1990 ->
+// 1157, 64 at k = 32 2400 -> 1404.  HBM is the floor at 754; the SM's issue
 // slots set the pace (expansion ~2000 of ~3900 warp instructions a tile).
 #include <algorithm>
 #include <cstring>
